@@ -155,21 +155,24 @@ struct PairPops {
                                               int x0, int xm, int xp, int y, int ym, int yp,
                                               float inv_scale, F2 (&f)[9], F2 (&gf)[5],
                                               F2 (&gs)[5]) {
-    const uint32_t r0 = (uint32_t)y * pi, rm = (uint32_t)ym * pi, rp = (uint32_t)yp * pi;
-    const uint32_t a = (uint32_t)x0, am = (uint32_t)xm, b = a + 1u, bp = (uint32_t)xp;
+    // one address per plane, the columns as offsets of it (Pops::pull)
+    const S* r0 = src + ((uint32_t)y * pi + (uint32_t)x0);
+    const S* rm = r0 + (int64_t)(ym - y) * pi;
+    const S* rp = r0 + (int64_t)(yp - y) * pi;
+    const int dm = xm - x0, dp = xp - x0;
     // i = 0, 2, 4: aligned pairs at rows y, y - 1, y + 1
     // i = 1, 5, 8 (e_x = +1): lanes from columns xm and x0
     // i = 3, 6, 7 (e_x = -1): lanes from columns x0 + 1 and xp
-    auto pair = [&](uint32_t k, uint32_t row) {
-      return PairIO<S>::ld2(src + (k * pl + row + a), inv_scale);
+    auto pair = [&](uint32_t k, const S* row) {
+      return PairIO<S>::ld2(row + (uint64_t)pl * k, inv_scale);
     };
-    auto left = [&](uint32_t k, uint32_t row) {
-      const uint32_t q = k * pl + row;
-      return PairIO<S>::ld11(src + (q + am), src + (q + a), inv_scale);
+    auto left = [&](uint32_t k, const S* row) {
+      const S* q = row + (uint64_t)pl * k;
+      return PairIO<S>::ld11(q + dm, q, inv_scale);
     };
-    auto right = [&](uint32_t k, uint32_t row) {
-      const uint32_t q = k * pl + row;
-      return PairIO<S>::ld11(src + (q + b), src + (q + bp), inv_scale);
+    auto right = [&](uint32_t k, const S* row) {
+      const S* q = row + (uint64_t)pl * k;
+      return PairIO<S>::ld11(q + 1, q + dp, inv_scale);
     };
     f[0] = pair(0, r0);
     f[1] = left(1, r0);
@@ -196,18 +199,19 @@ struct PairPops {
                                                float scale, const F2 (&f)[9], const F2 (&gf)[5],
                                                const F2 (&gs)[5], uint32_t seed_pair,
                                                uint32_t seed_step) {
+    S* const d = dst + off;
     if constexpr (Codec<S, float>::kStochastic) {
       RandomBits rb(seed_pair, seed_step);
 #pragma unroll
       for (int i = 0; i < 19; ++i) {
         const F2 v = i < 9 ? f[i] : (i < 14 ? gf[i - 9] : gs[i - 14]);
-        PairIO<S>::st2(dst + ((uint32_t)i * pl + off), v, scale, rb.next());
+        PairIO<S>::st2(d + (uint64_t)pl * (uint32_t)i, v, scale, rb.next());
       }
     } else {
 #pragma unroll
       for (int i = 0; i < 19; ++i) {
         const F2 v = i < 9 ? f[i] : (i < 14 ? gf[i - 9] : gs[i - 14]);
-        PairIO<S>::st2(dst + ((uint32_t)i * pl + off), v, scale, 0u);
+        PairIO<S>::st2(d + (uint64_t)pl * (uint32_t)i, v, scale, 0u);
       }
     }
   }
