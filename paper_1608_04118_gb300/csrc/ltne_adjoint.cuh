@@ -87,7 +87,7 @@ LTNE_HD void macros_adjoint(const NodeParams<C>& P, const Medium<C>& md, const C
   // ---- forward recomputation
   const C sgf = (gf[0] + gf[1]) + (gf[2] + gf[3]) + gf[4];
   const C sgs = (gs[0] + gs[1]) + (gs[2] + gs[3]) + gs[4];
-  const C cq = C(0.5) * (P.qf - P.qs);
+  const C cq = P.half_dq;
   const C D = ((sgf - sgs) + cq) * md.inv_1d;
   const C Srf = P.qf - md.a * D;
   const C dTf = sgf + C(0.5) * Srf;
@@ -198,39 +198,39 @@ LTNE_HD void collide_adjoint(const NodeParams<C>& P, const Medium<C>& md, const 
   const C ax = (A[5] - A[6]) + (A[8] - A[7]);
   const C ay = (A[5] - A[7]) + (A[6] - A[8]);
   // divisions by the small integers of D as in the forward collision
-  const C msb0 = div_small<C>(A[0] + sa + sd, C(9), C(1.0 / 9.0));
-  const C msb1 = div_small<C>(C(-4) * A[0] - sa + C(2) * sd, C(36), C(1.0 / 36.0));
-  const C msb2 = div_small<C>(C(4) * A[0] - C(2) * sa + sd, C(36), C(1.0 / 36.0));
-  const C msb3 = div_small<C>((A[1] - A[3]) + ax, C(6), C(1.0 / 6.0));
-  const C msb4 = div_small<C>(C(-2) * (A[1] - A[3]) + ax, C(12), C(1.0 / 12.0));
-  const C msb5 = div_small<C>((A[2] - A[4]) + ay, C(6), C(1.0 / 6.0));
-  const C msb6 = div_small<C>(C(-2) * (A[2] - A[4]) + ay, C(12), C(1.0 / 12.0));
+  const C msb0 = div_small<9, C>(A[0] + sa + sd);
+  const C msb1 = div_small<36, C>(C(-4) * A[0] - sa + C(2) * sd);
+  const C msb2 = div_small<36, C>(C(4) * A[0] - C(2) * sa + sd);
+  const C msb3 = div_small<6, C>((A[1] - A[3]) + ax);
+  const C msb4 = div_small<12, C>(C(-2) * (A[1] - A[3]) + ax);
+  const C msb5 = div_small<6, C>((A[2] - A[4]) + ay);
+  const C msb6 = div_small<12, C>(C(-2) * (A[2] - A[4]) + ay);
   const C msb7 = ((A[1] - A[2]) + (A[3] - A[4])) * C(0.25);
   const C msb8 = ((A[5] - A[6]) + (A[7] - A[8])) * C(0.25);
 
   mb.drho += msb0;
   const C m1_b = (C(1) - P.s_e) * msb1;
   const C meq1_b = P.s_e * msb1;
-  C S1_b = (C(1) - C(0.5) * P.s_e) * msb1;
+  C S1_b = P.half_e * msb1;
   const C m2_b = (C(1) - P.s_eps) * msb2;
   const C meq2_b = P.s_eps * msb2;
-  S1_b -= (C(1) - C(0.5) * P.s_eps) * msb2;
+  S1_b -= P.half_eps * msb2;
   mb.jx += msb3;
   C rFx_b = msb3;
   const C m4_b = (C(1) - P.s_q) * msb4;
   const C rux_b = -P.s_q * msb4;
-  rFx_b -= (C(1) - C(0.5) * P.s_q) * msb4;
+  rFx_b -= P.half_q * msb4;
   mb.jy += msb5;
   C rFy_b = msb5;
   const C m6_b = (C(1) - P.s_q) * msb6;
   const C ruy_b = -P.s_q * msb6;
-  rFy_b -= (C(1) - C(0.5) * P.s_q) * msb6;
+  rFy_b -= P.half_q * msb6;
   const C m7_b = (C(1) - P.s_nu) * msb7;
   const C meq7_b = P.s_nu * msb7;
-  const C S7_b = (C(1) - C(0.5) * P.s_nu) * msb7;
+  const C S7_b = P.half_nu * msb7;
   const C m8_b = (C(1) - P.s_nu) * msb8;
   const C meq8_b = P.s_nu * msb8;
-  const C S8_b = (C(1) - C(0.5) * P.s_nu) * msb8;
+  const C S8_b = P.half_nu * msb8;
 
   // equilibrium and forcing moments -> macroscopic values
   mb.drho += C(-2) * meq1_b + meq2_b;
@@ -267,10 +267,10 @@ LTNE_HD void collide_adjoint(const NodeParams<C>& P, const Medium<C>& md, const 
   // ---- temperatures.  ns_b = D_N^-1 N go_b.
   {
     const C* B = gfo_b;
-    const C nb0 = div_small<C>((B[0] + B[1]) + (B[2] + B[3]) + B[4], C(5), C(0.2));
+    const C nb0 = div_small<5, C>((B[0] + B[1]) + (B[2] + B[3]) + B[4]);
     const C nb1 = (B[1] - B[3]) * C(0.5);
     const C nb2 = (B[2] - B[4]) * C(0.5);
-    const C nb3 = div_small<C>(C(-4) * B[0] + ((B[1] + B[2]) + (B[3] + B[4])), C(20), C(0.05));
+    const C nb3 = div_small<20, C>(C(-4) * B[0] + ((B[1] + B[2]) + (B[3] + B[4])));
     const C nb4 = ((B[1] - B[2]) + (B[3] - B[4])) * C(0.25);
     const C Tf = P.T0 + m.dTf;
     mb.sgf += nb0;
@@ -290,7 +290,7 @@ LTNE_HD void collide_adjoint(const NodeParams<C>& P, const Medium<C>& md, const 
     }
     const C n3_b = (C(1) - P.zeta_e) * nb3;
     mb.dTf += P.zeta_e * P.c3 * nb3;
-    mb.Srf += (C(1) - C(0.5) * P.zeta_e) * P.c3 * nb3;
+    mb.Srf += P.c3_f * nb3;
     const C n4_b = (C(1) - P.zeta_nu) * nb4;
     gf_b[0] += C(-4) * n3_b;
     gf_b[1] += n1_b + n3_b + n4_b;
@@ -300,10 +300,10 @@ LTNE_HD void collide_adjoint(const NodeParams<C>& P, const Medium<C>& md, const 
   }
   {
     const C* B = gso_b;
-    const C nb0 = div_small<C>((B[0] + B[1]) + (B[2] + B[3]) + B[4], C(5), C(0.2));
+    const C nb0 = div_small<5, C>((B[0] + B[1]) + (B[2] + B[3]) + B[4]);
     const C nb1 = (B[1] - B[3]) * C(0.5);
     const C nb2 = (B[2] - B[4]) * C(0.5);
-    const C nb3 = div_small<C>(C(-4) * B[0] + ((B[1] + B[2]) + (B[3] + B[4])), C(20), C(0.05));
+    const C nb3 = div_small<20, C>(C(-4) * B[0] + ((B[1] + B[2]) + (B[3] + B[4])));
     const C nb4 = ((B[1] - B[2]) + (B[3] - B[4])) * C(0.25);
     mb.sgs += nb0;
     mb.Srs += nb0;
@@ -311,7 +311,7 @@ LTNE_HD void collide_adjoint(const NodeParams<C>& P, const Medium<C>& md, const 
     const C n2_b = (C(1) - P.eta_a) * nb2;
     const C n3_b = (C(1) - P.eta_e) * nb3;
     mb.dTs += P.eta_e * P.c3 * nb3;
-    mb.Srs += (C(1) - C(0.5) * P.eta_e) * P.c3 * nb3;
+    mb.Srs += P.c3_s * nb3;
     const C n4_b = (C(1) - P.eta_nu) * nb4;
     gs_b[0] += C(-4) * n3_b;
     gs_b[1] += n1_b + n3_b + n4_b;
