@@ -228,8 +228,11 @@ size_t ltne_state_bytes(const ltne_handle* h);
 int ltne_get_state(ltne_handle* h, void* host, size_t bytes);
 int ltne_set_state(ltne_handle* h, const void* host, size_t bytes);
 
-/* Number of step-kernel launches issued by this handle so far. */
+/* Number of time steps issued as step-kernel launches by this handle so far:
+   one per step, also where one launch advances two (see ltne_set_schedule).
+   ltne_kernel_launch_count: the launches themselves. */
 int64_t ltne_launch_count(const ltne_handle* h);
+int64_t ltne_kernel_launch_count(const ltne_handle* h);
 
 /* Launch schedule of the step kernel (no counterpart in the paper, which
    prescribes no implementation): blocks of block_x x block_y threads
@@ -241,8 +244,11 @@ int64_t ltne_launch_count(const ltne_handle* h);
    nodes_per_thread the block shape changes no bit.  Defaults: 32 x 4 with
    two nodes per thread for FP16 / BF16 lattices of 2^20 nodes or more,
    128 x 1 with two for FP32 lattices of 2^22 nodes or more, 64 x 2 with
-   one otherwise (and always for FP64).  May be called at any time between
-   steps.
+   one otherwise (and always for FP64).  With two nodes per thread, cavity
+   walls and no local h_v, lattices of 2^22 nodes or more (FP32) or 2^24
+   (16-bit storage) advance two steps per launch, in strips that do not
+   depend on the block shape; the results are the same bits.  May be called
+   at any time between steps.
    LTNE_ERR_INVALID_ARG for other schedules. */
 int ltne_set_schedule(ltne_handle* h, int32_t block_x, int32_t block_y,
                       int32_t nodes_per_thread);

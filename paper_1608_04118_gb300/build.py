@@ -63,7 +63,8 @@ def kernel_source_hash() -> str:
     step kernel (used to tell whether stored profiler counters still
     describe the current kernel)."""
     h = hashlib.sha256()
-    names = ["ltne_node.cuh", "ltne_step_impl.cuh", "ltne_pair.cuh", "ltne_internal.h"] + sorted(
+    names = ["ltne_node.cuh", "ltne_step_impl.cuh", "ltne_pair.cuh", "ltne_march.cuh",
+             "ltne_internal.h"] + sorted(
         os.path.basename(f) for f in glob.glob(os.path.join(CSRC, "step_*.cu")))
     for n in names:
         with open(os.path.join(CSRC, n)) as fh:

@@ -523,15 +523,30 @@ LatticeArgs lattice_args(const ltne_handle* h, int src_buf, int write_macros) {
   return a;
 }
 
+// Time steps one launch may advance on this handle: two where k_step2_pair
+// (ltne_march.cuh) is the faster form.  Its strips and segments need enough
+// rows of waves to fill the GPU: FP32 from 2^22 nodes (2048^2 96 -> 84 us a
+// step; 1024^2 27 -> 30), 16-bit storage from 2^24 (4096^2 FP16 303 -> 288;
+// 2048^2 81 -> 90).
+int steps_per_launch(const ltne_handle* h) {
+  const int64_t nodes = (int64_t)h->p.nx * h->p.ny;
+  const bool march = h->shape.pair && !h->shape.tma && !h->slab && !h->p.hv_local &&
+                     h->p.bc == LTNE_BC_CAVITY &&
+                     nodes >= (int64_t)1 << (h->p.storage == LTNE_F32 ? 22 : 24);
+  return march ? 2 : 1;
+}
+
 cudaError_t launch_step(ltne_handle* h, int src_buf, int write_macros, cudaStream_t st,
-                        bool chained = false) {
+                        bool chained = false, int steps = 1) {
   LatticeArgs a = lattice_args(h, src_buf, write_macros);
   a.chained = chained ? 1 : 0;
+  StepShape shape = h->shape;
+  shape.two = steps == 2;
   switch (h->p.storage) {
-    case LTNE_F64: return launch_step_f64(a, h->P, h->shape, st);
-    case LTNE_F32: return launch_step_f32(a, h->P, h->shape, st);
-    case LTNE_F16DEV: return launch_step_f16(a, h->P, h->shape, st);
-    default: return launch_step_bf16(a, h->P, h->shape, st);
+    case LTNE_F64: return launch_step_f64(a, h->P, shape, st);
+    case LTNE_F32: return launch_step_f32(a, h->P, shape, st);
+    case LTNE_F16DEV: return launch_step_f16(a, h->P, shape, st);
+    default: return launch_step_bf16(a, h->P, shape, st);
   }
 }
 
@@ -560,8 +575,9 @@ cudaError_t build_graph(ltne_handle* h, int parity) {
   if (e != cudaSuccess) return e;
   int b = parity;
   cudaError_t le = cudaSuccess;
-  for (int k = 0; k < kGraphSteps && le == cudaSuccess; ++k) {
-    le = launch_step(h, b, 0, h->cap_stream, k > 0);
+  const int per = steps_per_launch(h);
+  for (int k = 0; k < kGraphSteps && le == cudaSuccess; k += per) {
+    le = launch_step(h, b, 0, h->cap_stream, k > 0, per);
     b ^= 1;
   }
   cudaGraph_t g = nullptr;
@@ -1020,22 +1036,22 @@ int ltne_step(ltne_handle* h, int64_t n) {
     plain -= kGraphSteps;
     h->step += kGraphSteps;
     h->launches += kGraphSteps;
+    h->fused += kGraphSteps - kGraphSteps / steps_per_launch(h);
   }
   bool chained = false;  // the stream's last operation is a step kernel of this call
-  for (; plain > 0; --plain) {
-    e = launch_step(h, h->cur, 0, h->stream, chained);
+  for (int64_t left = plain + 1; left > 0;) {
+    int per = steps_per_launch(h);
+    if (left % per) per = 1;  // an odd step first
+    left -= per;
+    if (left == 0) begin_macro_write(h);  // the last step writes the fields
+    e = launch_step(h, h->cur, left == 0, h->stream, chained, per);
     if (e != cudaSuccess) return fail_cuda(e);
     chained = true;
     h->cur ^= 1;
-    ++h->step;
-    ++h->launches;
+    h->step += per;
+    h->launches += per;
+    h->fused += per - 1;
   }
-  begin_macro_write(h);  // the last step writes the fields
-  e = launch_step(h, h->cur, 1, h->stream, chained);
-  if (e != cudaSuccess) return fail_cuda(e);
-  h->cur ^= 1;
-  ++h->step;
-  ++h->launches;
   return LTNE_OK;
 }
 
@@ -1203,6 +1219,7 @@ int ltne_set_state(ltne_handle* h, const void* host, size_t bytes) {
 }
 
 int64_t ltne_launch_count(const ltne_handle* h) { return h ? h->launches : 0; }
+int64_t ltne_kernel_launch_count(const ltne_handle* h) { return h ? h->launches - h->fused : 0; }
 
 int ltne_set_schedule(ltne_handle* h, int32_t block_x, int32_t block_y,
                       int32_t nodes_per_thread) {

@@ -36,7 +36,8 @@ struct ltne_handle {
   int msnap = -1;           // macro set holding the snapshot (-1: none yet)
   float enc_scale = 1.0f;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  int64_t launches = 0;
+  int64_t launches = 0;  // time steps issued as step-kernel launches
+  int64_t fused = 0;     // of these, steps that shared a launch with the one before
   int32_t adj_sched = 0;  // LTNE_ADJ_*
   // two pinned host buffers that stage whole fields in and out (allocated
   // at the first set_fields / get_fields, freed by ltne_destroy), with an

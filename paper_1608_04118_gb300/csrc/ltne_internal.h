@@ -76,12 +76,14 @@ cudaError_t launch_kernel(bool chained, void (*k)(KArgs...), dim3 grid, dim3 blo
 // Launch configuration of the step kernel: a block of bx x by threads,
 // each advancing one node or (pair = 1, FP32 arithmetic only, at most
 // kPairBlockThreads threads per block) two neighbouring nodes of a row.
+constexpr int kSMs = 152;  // streaming multiprocessors of a GB300
 constexpr int kPairBlockThreads = 128;
 struct StepShape {
   int bx = 64;
   int by = 2;
   int pair = 0;
   int tma = 0;  // two nodes per thread from TMA-staged tiles (cavity walls only)
+  int two = 0;  // this launch advances two time steps
 };
 
 // Per-storage-type launchers (one translation unit each).

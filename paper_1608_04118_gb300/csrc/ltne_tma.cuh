@@ -31,7 +31,7 @@
 
 #include <mutex>
 
-#include "ltne_pair.cuh"
+#include "ltne_march.cuh"
 
 namespace ltne {
 
@@ -332,6 +332,7 @@ cudaError_t launch_step_tma_t(const LatticeArgs& a, const NodeParams<double>& Pd
   namespace ltne {                                                                             \
   cudaError_t launch_step_##tag(const LatticeArgs& a, const NodeParams<double>& P,             \
                                 StepShape s, cudaStream_t st) {                                \
+    if (s.two) return launch_step2_pair_t<S>(a, P, st);                                        \
     return s.tma    ? launch_step_tma_t<S>(a, P, s, st)                                       \
            : s.pair ? launch_step_pair_t<S>(a, P, s, st)                                      \
                     : launch_step_t<S, float>(a, P, s, st);                                   \

@@ -90,6 +90,7 @@ SIGNATURES = {
     "ltne_get_state": (C.c_int, [_vp, _vp, C.c_size_t]),
     "ltne_set_state": (C.c_int, [_vp, _vp, C.c_size_t]),
     "ltne_launch_count": (C.c_int64, [_vp]),
+    "ltne_kernel_launch_count": (C.c_int64, [_vp]),
     "ltne_set_schedule": (C.c_int, [_vp, C.c_int32, C.c_int32, C.c_int32]),
     "ltne_get_schedule": (C.c_int, [_vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                     C.POINTER(C.c_int32)]),
@@ -260,6 +261,10 @@ def ltne_set_state(h, blob: bytes):
 
 def ltne_launch_count(h) -> int:
     return int(_lib().ltne_launch_count(h))
+
+
+def ltne_kernel_launch_count(h) -> int:
+    return int(_lib().ltne_kernel_launch_count(h))
 
 
 def ltne_set_schedule(h, block_x, block_y, nodes_per_thread):
@@ -478,6 +483,11 @@ class Cavity:
     @property
     def launches(self):
         return ltne_launch_count(self.h)
+
+    @property
+    def kernel_launches(self):
+        """Step-kernel launches (a launch may advance two steps)."""
+        return ltne_kernel_launch_count(self.h)
 
     def set_schedule(self, block_x, block_y, nodes_per_thread):
         """Block shape and nodes per thread (1, or 2 in paired FP32) of the
