@@ -20,6 +20,7 @@
 #include "ltne.h"
 #include "ltne_internal.h"
 #include "ltne_handle.h"
+#include "ltne_tile.cuh"
 
 using namespace ltne;
 
@@ -523,17 +524,23 @@ LatticeArgs lattice_args(const ltne_handle* h, int src_buf, int write_macros) {
   return a;
 }
 
-// Time steps one launch may advance on this handle: two where k_step2_pair
-// (ltne_march.cuh) is the faster form.  Its strips and segments need enough
-// rows of waves to fill the GPU: FP32 from 2^22 nodes (2048^2 96 -> 84 us a
-// step; 1024^2 27 -> 30), 16-bit storage from 2^24 (4096^2 FP16 303 -> 288;
-// 2048^2 81 -> 90).
+// Time steps one launch may advance on this handle (a power of two, so that
+// the launches of a captured graph keep the A-B parity).  Two nodes per
+// thread: two where k_step2_pair (ltne_march.cuh) is the faster form.  Its
+// strips and segments need enough rows of waves to fill the GPU: FP32 from
+// 2^22 nodes (2048^2 96 -> 84 us a step; 1024^2 27 -> 30), 16-bit storage from
+// 2^24 (4096^2 FP16 303 -> 288; 2048^2 81 -> 90).  One node per thread, FP32
+// arithmetic: four where one block per SM holds the lattice in tiles of
+// k_step_tile (ltne_tile.cuh; up to about 200 x 200: 192^2 2.37 -> 2.18; with
+// two blocks per SM 256^2 2.88 -> 2.95).
 int steps_per_launch(const ltne_handle* h) {
-  const int64_t nodes = (int64_t)h->p.nx * h->p.ny;
-  const bool march = h->shape.pair && !h->shape.tma && !h->slab && !h->p.hv_local &&
-                     h->p.bc == LTNE_BC_CAVITY &&
-                     nodes >= (int64_t)1 << (h->p.storage == LTNE_F32 ? 22 : 24);
-  return march ? 2 : 1;
+  const ltne_params& p = h->p;
+  if (h->slab || h->shape.tma || p.bc != LTNE_BC_CAVITY || p.storage == LTNE_F64) return 1;
+  if (h->shape.pair) {
+    const int64_t nodes = (int64_t)p.nx * p.ny;
+    return !p.hv_local && nodes >= (int64_t)1 << (p.storage == LTNE_F32 ? 22 : 24) ? 2 : 1;
+  }
+  return h->shape.tiles.ntx ? kTileSteps : 1;
 }
 
 cudaError_t launch_step(ltne_handle* h, int src_buf, int write_macros, cudaStream_t st,
@@ -541,7 +548,7 @@ cudaError_t launch_step(ltne_handle* h, int src_buf, int write_macros, cudaStrea
   LatticeArgs a = lattice_args(h, src_buf, write_macros);
   a.chained = chained ? 1 : 0;
   StepShape shape = h->shape;
-  shape.two = steps == 2;
+  shape.steps = steps;
   switch (h->p.storage) {
     case LTNE_F64: return launch_step_f64(a, h->P, shape, st);
     case LTNE_F32: return launch_step_f32(a, h->P, shape, st);
@@ -989,6 +996,7 @@ int ltne_create(const ltne_params* p, void* cuda_stream, ltne_handle** out) {
   // by the latency of one thread's work (64 x 2 against 128 x 2: 40.5
   // against 38.3 GLUPS at 512^2 FP32, 34.2 against 32.2 FP16, equal at
   // 256^2 and in FP64).
+  h->shape.tiles = plan_tiles(p->nx, p->ny);
   const int64_t nodes = (int64_t)p->nx * p->ny;
   if ((p->storage == LTNE_F16DEV || p->storage == LTNE_BF16DEV) && nodes >= ((int64_t)1 << 20)) {
     h->shape.bx = 32;
@@ -1041,7 +1049,7 @@ int ltne_step(ltne_handle* h, int64_t n) {
   bool chained = false;  // the stream's last operation is a step kernel of this call
   for (int64_t left = plain + 1; left > 0;) {
     int per = steps_per_launch(h);
-    if (left % per) per = 1;  // an odd step first
+    if (left % per) per = (int)(left % per);  // the remainder first
     left -= per;
     if (left == 0) begin_macro_write(h);  // the last step writes the fields
     e = launch_step(h, h->cur, left == 0, h->stream, chained, per);

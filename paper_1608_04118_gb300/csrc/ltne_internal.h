@@ -78,12 +78,18 @@ cudaError_t launch_kernel(bool chained, void (*k)(KArgs...), dim3 grid, dim3 blo
 // kPairBlockThreads threads per block) two neighbouring nodes of a row.
 constexpr int kSMs = 152;  // streaming multiprocessors of a GB300
 constexpr int kPairBlockThreads = 128;
+// Tiles of k_step_tile (plan_tiles); ntx = 0: the lattice is too large for it.
+struct TilePlan {
+  int ntx = 0, nty = 0, threads = 0;
+};
+
 struct StepShape {
   int bx = 64;
   int by = 2;
   int pair = 0;
   int tma = 0;  // two nodes per thread from TMA-staged tiles (cavity walls only)
-  int two = 0;  // this launch advances two time steps
+  int steps = 1;  // time steps this launch advances (steps_per_launch)
+  TilePlan tiles; // of launches that advance several steps with one node per thread
 };
 
 // Per-storage-type launchers (one translation unit each).

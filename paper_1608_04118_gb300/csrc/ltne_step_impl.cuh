@@ -138,6 +138,42 @@ __device__ __forceinline__ void store_macros(C* __restrict__ mac, int64_t plane,
   mac[4 * pl + off] = m.dTs;
 }
 
+// From a node's pulled values to its post-collision values, in place: wall
+// rebuild (kind >= 0: the values were pulled around the interior neighbour at
+// offset noff), macroscopic values m, collision.  um, umn: |u| of the previous
+// state at the node and at the neighbour (read for the local h_v only).
+// kind: -1 interior, 0 hot wall, 1 cold wall, 2 adiabatic / no-slip row.
+template <typename C, int BC>
+__device__ __forceinline__ void update_node(const NodeParams<C>& P,
+                                            const C* __restrict__ phi_field, const uint32_t off,
+                                            const uint32_t noff, const int kind, const C* um,
+                                            const C* umn, const int64_t plane,
+                                            C* __restrict__ pre_out, C (&f)[9], C (&gf)[5],
+                                            C (&gs)[5], Macro<C>& m) {
+  if (BC != BC_PERIODIC && kind >= 0) {
+    Medium<C> mdn = phi_field ? medium_at<C>(P, phi_field[noff]) : P.um;
+    if (P.hv_local) set_exchange<C>(mdn, hv_local_at<C>(P, *umn));
+    Macro<C> mn;
+    macros<C>(P, mdn, f, gf, gs, mn);
+    C dTwf = mn.dTf, dTws = mn.dTs;  // adiabatic: the neighbour's temperature
+    if (kind == 0) dTwf = dTws = P.dT_hot;
+    if (kind == 1) dTwf = dTws = P.dT_cold;
+    nee<C>(P, mn, dTwf, dTws, f, gf, gs);
+  }
+  if (pre_out) {  // record the pre-collision state (reverse-mode recomputation)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) pre_out[(int64_t)i * plane + off] = f[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) pre_out[(int64_t)(9 + i) * plane + off] = gf[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) pre_out[(int64_t)(14 + i) * plane + off] = gs[i];
+  }
+  Medium<C> md = phi_field ? medium_at<C>(P, phi_field[off]) : P.um;
+  if (P.hv_local) set_exchange<C>(md, hv_local_at<C>(P, *um));
+  macros<C>(P, md, f, gf, gs, m);
+  collide<C>(P, m, f, gf, gs);
+}
+
 // One node (x, y) of one time step: pull, wall rebuild, macroscopic values,
 // collision, store.  Shared by the single-lattice and the batched kernels.
 template <typename S, typename C, int BC>
@@ -153,7 +189,7 @@ __device__ __forceinline__ void step_node(const S* __restrict__ src, S* __restri
                                           const int slab_walls = 0) {
   // Wall classification and the node whose neighbourhood is pulled.
   int cx = x, cy = y;
-  int kind = -1;  // -1 interior, 0 hot wall, 1 cold wall, 2 adiabatic / no-slip row
+  int kind = -1;
   if (BC == BC_CAVITY || BC == BC_SLAB) {
     const bool ylo = (BC == BC_CAVITY || (slab_walls & SLAB_LO_WALL)) && y == 0;
     const bool yhi = (BC == BC_CAVITY || (slab_walls & SLAB_HI_WALL)) && y == ny - 1;
@@ -186,32 +222,12 @@ __device__ __forceinline__ void step_node(const S* __restrict__ src, S* __restri
   Pops<S, C>::pull(src, pitch, plane, cx, xm, xp, cy, ym, yp, inv_scale, f, gf, gs);
 
   const uint32_t off = (uint32_t)y * (uint32_t)pitch + (uint32_t)x;
-  if (BC != BC_PERIODIC && kind >= 0) {
-    const uint32_t noff = (uint32_t)cy * (uint32_t)pitch + (uint32_t)cx;
-    Medium<C> mdn = phi_field ? medium_at<C>(P, phi_field[noff]) : P.um;
-    if (P.hv_local) set_exchange<C>(mdn, hv_local_at<C>(P, um_in[noff]));
-    Macro<C> mn;
-    macros<C>(P, mdn, f, gf, gs, mn);
-    C dTwf = mn.dTf, dTws = mn.dTs;  // adiabatic: the neighbour's temperature
-    if (kind == 0) dTwf = dTws = P.dT_hot;
-    if (kind == 1) dTwf = dTws = P.dT_cold;
-    nee<C>(P, mn, dTwf, dTws, f, gf, gs);
-  }
-  if (pre_out) {  // record the pre-collision state (reverse-mode recomputation)
-#pragma unroll
-    for (int i = 0; i < 9; ++i) pre_out[(int64_t)i * plane + off] = f[i];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) pre_out[(int64_t)(9 + i) * plane + off] = gf[i];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) pre_out[(int64_t)(14 + i) * plane + off] = gs[i];
-  }
-  Medium<C> md = phi_field ? medium_at<C>(P, phi_field[off]) : P.um;
-  if (P.hv_local) set_exchange<C>(md, hv_local_at<C>(P, um_in[off]));
+  const uint32_t noff = (uint32_t)cy * (uint32_t)pitch + (uint32_t)cx;
   Macro<C> m;
-  macros<C>(P, md, f, gf, gs, m);
+  update_node<C, BC>(P, phi_field, off, noff, kind, um_in + off, um_in + noff, plane, pre_out, f,
+                     gf, gs, m);
   if (P.hv_local) um_out[off] = m.umag;  // u_m of Eq. 52 for the next state
   if (write_macros) store_macros<C>(mac, plane, off, m);
-  collide<C>(P, m, f, gf, gs);
   Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, (uint32_t)off, tick);
 }
 

@@ -32,6 +32,7 @@
 #include <mutex>
 
 #include "ltne_march.cuh"
+#include "ltne_tile.cuh"
 
 namespace ltne {
 
@@ -327,12 +328,15 @@ cudaError_t launch_step_tma_t(const LatticeArgs& a, const NodeParams<double>& Pd
 }  // namespace ltne
 
 // Launchers of a storage type with FP32 arithmetic: the schedule picks one
-// or two nodes per thread, and the staged or the direct-load two-node form.
+// or two nodes per thread, and the staged or the direct-load two-node form;
+// launches of several steps have kernels of their own.
 #define LTNE_DEFINE_FLOAT_LAUNCHERS(tag, S)                                                     \
   namespace ltne {                                                                             \
   cudaError_t launch_step_##tag(const LatticeArgs& a, const NodeParams<double>& P,             \
                                 StepShape s, cudaStream_t st) {                                \
-    if (s.two) return launch_step2_pair_t<S>(a, P, st);                                        \
+    if (s.steps > 1)                                                                           \
+      return s.pair ? launch_step2_pair_t<S>(a, P, st)                                         \
+                    : launch_step_tile_t<S, float>(a, P, s, st);                               \
     return s.tma    ? launch_step_tma_t<S>(a, P, s, st)                                       \
            : s.pair ? launch_step_pair_t<S>(a, P, s, st)                                      \
                     : launch_step_t<S, float>(a, P, s, st);                                   \
