@@ -826,7 +826,7 @@ int set_fields_impl(ltne_handle* h, const double* porosity, const double* rho, c
   return LTNE_OK;
 }
 
-int reduce_launch(ltne_handle* h) {
+int reduce_launch(ltne_handle* h, double* host_out) {
   const ltne_params& p = h->p;
   ReduceArgs a;
   a.mac = mac_cur(h);
@@ -844,6 +844,8 @@ int reduce_launch(ltne_handle* h) {
   a.sigma = p.sigma;
   a.qf = p.qf;
   a.qs = p.qs;
+  a.host_out = host_out;
+  a.err = reinterpret_cast<const int*>(h->ws + h->off_tick + 2 * sizeof(uint32_t));
   a.update_prev = 0;  // the snapshot is a whole macro set (see ltne_observables)
   a.blocks = h->red_blocks;
   a.is_double = h->ec == 8;
@@ -1070,18 +1072,13 @@ int ltne_observables(ltne_handle* h, ltne_obs* out) {
   cudaError_t e = cudaSuccess;
   e = ensure_pin_obs(h);
   if (e != cudaSuccess) return fail_cuda(e);
-  const int rr = reduce_launch(h);
+  // the accumulators and the device error word land in pinned memory: a
+  // staged step that gave up waiting for its tile reports here (the fields
+  // are then not trustworthy); the word is cleared
+  const int rr = reduce_launch(h, h->pin_obs);
   if (rr != LTNE_OK) return rr;
-  // the accumulators and the device error word in one read-back: a staged
-  // step that gave up waiting for its tile reports here (the fields are then
-  // not trustworthy); the word is cleared
-  int* errp = reinterpret_cast<int*>(h->pin_obs + NACC);
-  e = cudaMemcpyAsync(h->pin_obs, h->ws + h->off_out, NACC * sizeof(double),
-                      cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(errp, h->ws + h->off_tick + 2 * sizeof(uint32_t), sizeof(int),
-                        cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const int* errp = reinterpret_cast<const int*>(h->pin_obs + NACC);
+  e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return fail_cuda(e);
   double acc[NACC];
   for (int k = 0; k < NACC; ++k) acc[k] = h->pin_obs[k];

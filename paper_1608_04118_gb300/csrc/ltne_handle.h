@@ -59,7 +59,7 @@ struct ltne_handle {
   int slo = 0, shi = 0;    // halo row below / above (0 or 1)
   size_t off_halo[4] = {0, 0, 0, 0};  // send below, send above, receive below, above
   // pinned landing place of the observables' accumulators and the device
-  // error word (one asynchronous read-back per ltne_observables call)
+  // error word, written by the reduction's last kernel
   double* pin_obs = nullptr;
 };
 
@@ -78,6 +78,7 @@ int set_fields_impl(ltne_handle* h, const double* porosity, const double* rho, c
 // The handle's observables reduction into acc[NACC] (synchronises).
 int reduce_handle(ltne_handle* h, double* acc);
 // The same reduction, enqueued on the handle's stream only (the result in
-// the workspace's output slot).
-int reduce_launch(ltne_handle* h);
+// the workspace's output slot, and in host_out where that is given: NACC
+// accumulators and the device error word, see ReduceArgs).
+int reduce_launch(ltne_handle* h, double* host_out = nullptr);
 }  // namespace ltne

@@ -116,6 +116,10 @@ struct ReduceArgs {
   void* prev;        // 4 planes: ux, uy, Tf, Ts of the previous call
   double* partials;  // [blocks][NACC] scratch
   double* out;       // [NACC]
+  // page-locked host memory that also receives the accumulators and, after
+  // them, the int at err; or nullptr
+  double* host_out = nullptr;
+  const int* err = nullptr;
   int nx, ny;
   int64_t pitch, plane;
   double phi_u, sigma, qf, qs;

@@ -42,27 +42,18 @@ __device__ __forceinline__ C combine(int k, C a, C b) {
   return (k == A_MAXU || k == A_MAXDT) ? cmax(a, b) : a + b;
 }
 
-// Block-wide reduction of NACC accumulators per thread into acc of
-// thread 0 (fixed shuffle and warp order).
-__device__ void block_reduce(double (&acc)[NACC], double* sh /* [RB/32][NACC] */) {
+// Block-wide reduction of one value per thread, for accumulator k: the lanes
+// of a warp by strides 16 .. 1, then the warps in order; in thread 0.
+__device__ double block_reduce(int k, double v, double* sh /* [RB/32] */) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < NACC; ++k) {
-    double v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      v = combine<double>(k, v, __shfl_down_sync(0xffffffffu, v, o));
-    acc[k] = v;
-  }
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NACC; ++k) sh[warp * NACC + k] = acc[k];
+  for (int o = 16; o > 0; o >>= 1)
+    v = combine<double>(k, v, __shfl_down_sync(0xffffffffu, v, o));
+  if (lane == 0) sh[warp] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < RB / 32; ++w)
-#pragma unroll
-      for (int k = 0; k < NACC; ++k) acc[k] = combine<double>(k, acc[k], sh[w * NACC + k]);
-  }
+  if (threadIdx.x == 0)
+    for (int w = 1; w < RB / 32; ++w) v = combine<double>(k, v, sh[w]);
+  return v;
 }
 
 static_assert(A_NUF_H == 0 && A_NUS_H == 1 && A_NUF_C == 2 && A_NUS_C == 3 && A_MASS == 4,
@@ -178,12 +169,16 @@ __global__ void __launch_bounds__(RB) k_reduce_pass1(ReduceArgs a, int seg) {
 // q_cold = -1.5 T_c + 2 T(nx-2,y) - 0.5 T(nx-3,y) of one phase (their
 // deviation parts; the wall terms are added on the host), trapezoid rule in
 // y -- thread t taking rows or partials t, t + RB, ..., then the block tree.
+// A programmatic dependent of pass 1.  Bound: latency.  Each block reduces its
+// one accumulator (all 18 in every block kept the FP64 pipe, two lanes per SM,
+// busy for most of the pass), and the result goes to the caller's page-locked
+// host memory as well where that is given, with the device error word: no
+// copies after the kernel.  One ltne_observables call at 64^2: 50 us before,
+// 30 now (FP64 fields 72 and 49, 4096^2 FP32 149 and 139).
 template <typename C>
 __global__ void __launch_bounds__(RB) k_reduce_pass2(ReduceArgs a) {
-  __shared__ double sh[(RB / 32) * NACC];
-  double acc[NACC];
-#pragma unroll
-  for (int k = 0; k < NACC; ++k) acc[k] = 0.0;
+  __shared__ double sh[RB / 32];
+  grid_dep_wait();
   const int k = blockIdx.x;
   double v = 0.0;
   if (k >= A_MASS) {
@@ -203,9 +198,14 @@ __global__ void __launch_bounds__(RB) k_reduce_pass2(ReduceArgs a) {
       v += wy * (w1 * (double)row[c1] + w2 * (double)row[c2]);
     }
   }
-  acc[k] = v;
-  block_reduce(acc, sh);
-  if (threadIdx.x == 0) a.out[k] = acc[k];
+  v = block_reduce(k, v, sh);
+  if (threadIdx.x == 0) {
+    a.out[k] = v;
+    if (a.host_out) {
+      a.host_out[k] = v;
+      if (k == 0) *reinterpret_cast<int*>(a.host_out + NACC) = *a.err;
+    }
+  }
 }
 
 }  // namespace
@@ -225,11 +225,8 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t st) {
     k_reduce_pass1<float><<<grid, RB, 0, st>>>(a, seg);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (a.is_double)
-    k_reduce_pass2<double><<<NACC, RB, 0, st>>>(a);
-  else
-    k_reduce_pass2<float><<<NACC, RB, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(true, a.is_double ? k_reduce_pass2<double> : k_reduce_pass2<float>,
+                       dim3(NACC), dim3(RB), 0, st, a);
 }
 
 }  // namespace ltne
