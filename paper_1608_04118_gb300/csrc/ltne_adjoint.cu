@@ -153,37 +153,64 @@ __device__ __forceinline__ void fold_wall(const NodeParams<C>& P, const WallSour
 
 // Adds to the gathered adjoint q (pulled from y + e_i) the folds stored at
 // the wall nodes of each target next to a wall: its side-column node, its
-// bottom/top-row node, then the corner, in that order.
-template <typename C>
+// bottom/top-row node, then the corner, in that order.  kBatch: each of the
+// three reads all its values before it adds any, one round trip to L2 on the
+// reverse chain instead of one per direction (256^2 x 400 steps 4.55 -> 4.36 ms
+// before the rest was settled, 64^2 3.14 -> 2.89), for 19 registers more; the
+// builds short of them (1024^2, capped: 11.7 -> 12.2 ms) read and add direction
+// by direction.
+template <bool kBatch, typename C>
 __device__ __forceinline__ void add_wall_folds(const C* __restrict__ Lam, int x, int y, int nx,
                                                int ny, int64_t pitch, int64_t plane,
                                                C (&qf)[9], C (&qgf)[5], C (&qgs)[5]) {
   const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
+  // whether target i takes its fold k (0 side column, 1 row, 2 corner), and from where
+  auto fold_at = [&](int i, int k, int64_t& wo) {
     const int tx = x + ex[i], ty = y + ey[i];
-    if (tx < 1 || tx > nx - 2 || ty < 1 || ty > ny - 2) continue;
+    const bool in = tx >= 1 && tx <= nx - 2 && ty >= 1 && ty <= ny - 2;
     const bool cx = tx == 1 || tx == nx - 2, cy = ty == 1 || ty == ny - 2;
-    if (!cx && !cy) continue;
-    const int wx = (tx == 1) ? 0 : nx - 1, wy = (ty == 1) ? 0 : ny - 1;
-    int64_t wo[3];
-    bool wv[3];
-    wv[0] = cx;
-    wo[0] = (int64_t)ty * pitch + wx;
-    wv[1] = cy;
-    wo[1] = (int64_t)wy * pitch + tx;
-    wv[2] = cx && cy;
-    wo[2] = (int64_t)wy * pitch + wx;
+    const int wx = k == 1 ? tx : (tx == 1 ? 0 : nx - 1);
+    const int wy = k == 0 ? ty : (ty == 1 ? 0 : ny - 1);
+    wo = (int64_t)wy * pitch + wx;
+    return in && (k == 1 || cx) && (k == 0 || cy);
+  };
+  int64_t wo;
+  if constexpr (kBatch) {
+    const bool near_x = x <= 2 || x >= nx - 3, near_y = y <= 2 || y >= ny - 3;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      if (!wv[k]) continue;
-      qf[i] += Lam[(int64_t)i * plane + wo[k]];
-      if (i < 5) {
-        qgf[i] += Lam[(int64_t)(9 + i) * plane + wo[k]];
-        qgs[i] += Lam[(int64_t)(14 + i) * plane + wo[k]];
+      if (!((k == 1 || near_x) && (k == 0 || near_y))) continue;
+      C tf[9], tgf[5], tgs[5];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const bool v = fold_at(i, k, wo);
+        tf[i] = v ? Lam[(int64_t)i * plane + wo] : C(0);
+        if (i < 5) {
+          tgf[i] = v ? Lam[(int64_t)(9 + i) * plane + wo] : C(0);
+          tgs[i] = v ? Lam[(int64_t)(14 + i) * plane + wo] : C(0);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 9; ++i) qf[i] += tf[i];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        qgf[i] += tgf[i];
+        qgs[i] += tgs[i];
       }
     }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (!fold_at(i, k, wo)) continue;
+        qf[i] += Lam[(int64_t)i * plane + wo];
+        if (i < 5) {
+          qgf[i] += Lam[(int64_t)(9 + i) * plane + wo];
+          qgs[i] += Lam[(int64_t)(14 + i) * plane + wo];
+        }
+      }
   }
 }
 
@@ -233,14 +260,26 @@ __global__ void __launch_bounds__(256) k_adj_seed(const C* __restrict__ SN, C* _
 
 // R2: transposed streaming (gather from y + e_i) and transposed collision;
 // a wall node's thread then folds its result (R1) unless S_n is the initial
-// state (fold = 0), whose wall nodes were not rebuilt.  The fold raises the
-// kernel's registers (123 against 73 without it, FP32).  Two builds of the
-// same code: kCapped = false keeps them all (lattices that fit one wave,
-// where the kernel's time is one thread's latency); kCapped = true caps them
-// at 64, 1024 threads' worth per SM (FP32; larger lattices, where occupancy
-// hides the latency), spilling a few values to local memory.
+// state (fold = 0), whose wall nodes were not rebuilt.  Two builds of the same
+// code: kCapped = false for lattices that fit one wave, where the kernel's
+// time is one thread's latency; kCapped = true with registers capped at 80,
+// 768 threads per SM (FP32), for larger lattices, where occupancy hides it
+// (at 72 and 64 registers the spills cost more: 400^2 x 100 steps 2.82 and 2.70
+// against 2.56 ms).
+//
+// The one-wave build loads the recorded state, also a wall node's source,
+// before it waits for the previous reverse step, and lets the next step's
+// blocks start once its own adjoint is computed, so that their loads fill the
+// launch gap.  (The state was recorded a whole segment ago: no kernel that
+// this one is chained to writes it.)  At most 128 registers, four blocks per
+// SM: the 512 blocks of a 256^2 lattice are then one wave.  Whole calls of 400
+// steps, before -> now with this and the batched folds: 256^2 5.18 -> 4.41 ms,
+// 131 x 97 3.89 -> 3.22, 64^2 3.54 -> 2.92.  The macroscopic values formed before
+// the wait as well gave 4.36 at 256^2, but other contractions (dJ/dphi 2e-6
+// apart); on larger lattices what is held across the wait costs occupancy
+// (1024^2 12.0 -> 13.4 ms), so the capped build waits first.
 template <typename C, bool kCapped>
-__global__ void __launch_bounds__(256, (kCapped && sizeof(C) == 4) ? 4 : 1)
+__global__ void __launch_bounds__(128, sizeof(C) == 8 ? 1 : kCapped ? 6 : 4)
     k_adj_main(const C* __restrict__ Lam,
                                                   C* __restrict__ lam_out,
                                                   const C* __restrict__ S,
@@ -249,11 +288,22 @@ __global__ void __launch_bounds__(256, (kCapped && sizeof(C) == 4) ? 4 : 1)
                                                   C* __restrict__ wphib, const NodeParams<C> P,
                                                   int nx, int ny, int64_t pitch, int64_t plane,
                                                   int fold, const C* __restrict__ S_prev) {
-  grid_dep_wait();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= nx || y >= ny) return;
+  if (x >= nx || y >= ny) {
+    grid_dep_wait();
+    return;
+  }
   const int64_t off = (int64_t)y * pitch + x;
+  const bool wall = fold && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1);
+  WallSource<C> w;
+  C f[9], gf[5], gs[5], ph;
+  if (!kCapped) {
+    load19(S, plane, off, f, gf, gs);
+    ph = phi[off];
+    if (wall) load_wall_source(S, phi, x, y, nx, ny, pitch, plane, w);
+  }
+  grid_dep_wait();
   // one-wave build: this node's gradient accumulators, read here so that
   // their latency is not the last link of the chain below (the capped build
   // keeps its registers for the chain and reads them at the end)
@@ -285,19 +335,19 @@ __global__ void __launch_bounds__(256, (kCapped && sizeof(C) == 4) ? 4 : 1)
       qgs[i] = pulled ? Lam[(int64_t)(14 + i) * plane + toff] : C(0);
     }
   }
+  if (kCapped) {
+    load19(S, plane, off, f, gf, gs);
+    ph = phi[off];
+  }
   if (x <= 2 || x >= nx - 3 || y <= 2 || y >= ny - 3)
-    add_wall_folds(Lam, x, y, nx, ny, pitch, plane, qf, qgf, qgs);
-  const bool wall = fold && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1);
-  WallSource<C> w;
-  if (wall) load_wall_source(S, phi, x, y, nx, ny, pitch, plane, w);
-  C f[9], gf[5], gs[5];
-  load19(S, plane, off, f, gf, gs);
-  const C ph = phi[off];
+    add_wall_folds<!kCapped && sizeof(C) == 4>(Lam, x, y, nx, ny, pitch, plane, qf, qgf, qgs);
+  if (kCapped && wall) load_wall_source(S, phi, x, y, nx, ny, pitch, plane, w);
   const Medium<C> md = medium_at<C>(P, ph);
   C fb[9] = {}, gfb[5] = {}, gsb[5] = {};
   MediumBar<C> mdb;
   zero(mdb);
   collide_adjoint<C>(P, md, f, gf, gs, qf, qgf, qgs, fb, gfb, gsb, mdb);
+  if (!kCapped) grid_dep_trigger();
   C pb = C(0), hv = C(0);
   if (wall)
     fold_wall(P, w, fb, gfb, gsb, lam_out, wphib, plane, off, hv);

@@ -49,11 +49,15 @@ struct LatticeArgs {
 // memory; without the launch attribute the wait is a no-op.  Every thread
 // of a kernel that may be launched so executes it before any global access
 // or early return, so each grid completes only after its predecessor did.
-// No kernel triggers its dependents early (griddepcontrol.launch_dependents):
-// blocks of the next kernel parked on the SMs while a single-wave grid still
-// runs made the adjoint's chain 6-20 % slower at 256 x 256.
 __device__ __forceinline__ void grid_dep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Lets the next kernel's blocks start (they wait in grid_dep_wait() for this
+// grid's completion all the same).  Worth it where the next kernel has work
+// that does not depend on this one before its wait (k_adj_main); without such
+// work its parked blocks only take slots (6-20 % slower at 256 x 256).
+__device__ __forceinline__ void grid_dep_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Launch k with the programmatic-serialisation attribute when `chained`.

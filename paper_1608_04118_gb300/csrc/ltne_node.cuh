@@ -102,10 +102,10 @@ template <> LTNE_HD double cfma_<double>(double a, double b, double c) {
 // RN(1/D) and lo = RN(1/D - hi), and x hi + x lo with one fused rounding.  A
 // plain product with hi would add its bias at every step -- in FP32,
 // 6 RN(1/6) = 1 + 3e-8 would grow the momentum by that factor per step.  For
-// every D used here and every normal FP32 x the result is the correctly
-// rounded quotient (all 2^23 significands tried), the same bits as the
-// product corrected by the residual x - D q (an FMA more); in FP64 it is the
-// quotient to within 2^-53 (1 + 2^-52).
+// every D used here and every FP32 x from 1e-36 up (below, x lo loses bits) the
+// result is the correctly rounded quotient (all 2^23 significands tried), the
+// same bits as the product corrected by the residual x - D q (an FMA more); in
+// FP64 it is the quotient to within 2^-53 (1 + 2^-52).
 template <int D> struct InvSmall;
 #define LTNE_INV_SMALL(D, LO64)                                                        \
   template <> struct InvSmall<D> {                                                     \
