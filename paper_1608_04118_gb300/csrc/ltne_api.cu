@@ -162,8 +162,11 @@ void release_pinned(ltne_handle* h) {
   h->pin_bytes = 0;
 }
 
-cudaError_t ensure_pinned(ltne_handle* h, size_t row_bytes) {
-  const size_t bytes = std::max(row_bytes, kPinBytes);
+// Two buffers of at least `need` bytes each, and room for the five macro planes
+// of a lattice up to kPinBytes (page-locking 64 MB for a small lattice took
+// 2 ms of its first get_fields).
+cudaError_t ensure_pinned(ltne_handle* h, size_t need) {
+  const size_t bytes = std::max(need, std::min(kPinBytes, 5 * (size_t)h->plane * h->ec));
   if (h->pin_bytes >= bytes) return cudaSuccess;
   release_pinned(h);
   for (int k = 0; k < 2; ++k) {
@@ -698,7 +701,6 @@ int set_fields_impl(ltne_handle* h, const double* porosity, const double* rho, c
   // From here the device state is being replaced: a failure below leaves
   // the handle without fields until a set_fields call succeeds.
   h->fields_set = false;
-  drop_graphs(h);  // kernel arguments captured in graphs depend on the parameters
 
   // Zero the whole workspace first -- population buffers, porosity, both
   // macro sets, |u| planes, counters -- so that row and plane padding, which
@@ -1036,8 +1038,14 @@ int ltne_step(ltne_handle* h, int64_t n) {
   if (n == 0) return LTNE_OK;
   int64_t plain = n - 1;  // the last step also writes the macroscopic fields
   cudaError_t e;
+  // the lattice constants are arguments of the captured launches: a graph
+  // outlives set_fields as long as they are the same (a capture and its
+  // instantiation took 100 us of every run started anew)
+  if ((h->graph[0] || h->graph[1]) && memcmp(&h->graph_P, &h->P, sizeof(h->P)) != 0)
+    drop_graphs(h);
   while (plain >= kGraphSteps) {
     if (!h->graph[h->cur]) {
+      memcpy(&h->graph_P, &h->P, sizeof(h->P));
       e = build_graph(h, h->cur);
       if (e != cudaSuccess) return fail_cuda(e);
     }
@@ -1113,6 +1121,34 @@ int ltne_get_fields(ltne_handle* h, double* rho, double* ux, double* uy, double*
                                           hp, h->stream);
     const cudaError_t es = cudaStreamSynchronize(h->stream);
     return fail_cuda(e != cudaSuccess ? e : es);
+  }
+  // small lattices: all five planes in one copy, then converted row by row
+  const size_t all = 5 * (size_t)h->plane * h->ec;
+  if (all <= kPinBytes) {
+    cudaError_t e = ensure_pinned(h, all);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->pin[0], mac_cur(h), all, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return fail_cuda(e);
+    for (int k = 0; k < 5; ++k) {
+      if (!dst[k]) continue;
+      const double ref = (k == 0) ? 1.0 : (k >= 3 ? p.T_ref : 0.0);  // planes hold deviations
+      double* out = dst[k];
+      const int64_t pitch = h->pitch;
+      auto convert = [&](const auto* t) {  // rows lo .. hi - 1
+        host_chunks(
+            p.ny,
+            [&](int, int64_t lo, int64_t hi) {
+              for (int64_t y = lo; y < hi; ++y)
+                for (int64_t x = 0; x < nx; ++x) out[y * nx + x] = ref + (double)t[y * pitch + x];
+            },
+            (((int64_t)1 << 18) + nx - 1) / nx);
+      };
+      const char* plane = h->pin[0] + (size_t)k * h->plane * h->ec;
+      if (h->ec == 8) convert(reinterpret_cast<const double*>(plane));
+      else convert(reinterpret_cast<const float*>(plane));
+    }
+    return LTNE_OK;
   }
   for (int k = 0; k < 5; ++k) {
     if (!dst[k]) continue;

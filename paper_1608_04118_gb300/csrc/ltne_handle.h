@@ -36,6 +36,7 @@ struct ltne_handle {
   int msnap = -1;           // macro set holding the snapshot (-1: none yet)
   float enc_scale = 1.0f;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  ltne::NodeParams<double> graph_P{};  // the lattice constants the graphs were captured with
   int64_t launches = 0;  // time steps issued as step-kernel launches
   int64_t fused = 0;     // of these, steps that shared a launch with the one before
   int32_t adj_sched = 0;  // LTNE_ADJ_*
