@@ -98,19 +98,19 @@ template <> LTNE_HD double cfma_<double>(double a, double b, double c) {
   return fma(a, b, c);
 }
 
-// x / D for a small integer D: the reciprocal as a sum of two numbers, hi =
-// RN(1/D) and lo = RN(1/D - hi), and x hi + x lo with one fused rounding.  A
-// plain product with hi would add its bias at every step -- in FP32,
-// 6 RN(1/6) = 1 + 3e-8 would grow the momentum by that factor per step.  For
-// every D used here and every FP32 x from 1e-36 up (below, x lo loses bits) the
-// result is the correctly rounded quotient (all 2^23 significands tried), the
-// same bits as the product corrected by the residual x - D q (an FMA more); in
-// FP64 it is the quotient to within 2^-53 (1 + 2^-52).
+// x / D for a small integer D.  FP32: the product with hi = RN(1/D) and one
+// residual correction (r = x - D q is exact in an FMA), which removes the
+// systematic bias that the plain product would add at every step -- in FP32,
+// 6 RN(1/6) = 1 + 3e-8 would grow the momentum by that factor per step.  FP64:
+// the reciprocal as hi + lo, lo = RN(1/D - hi), and x hi + x lo with one fused
+// rounding, an operation less: the quotient to within 2^-53 (1 + 2^-52).  (In
+// FP32 that form gives the same bits for every normal significand, but not
+// below 1e-36, where x lo loses bits; a run from exact rest carries that into
+// the last place of its fields, so FP32 keeps the correction.)
 template <int D> struct InvSmall;
-#define LTNE_INV_SMALL(D, LO64)                                                        \
-  template <> struct InvSmall<D> {                                                     \
-    static constexpr double hi = 1.0 / D, lo64 = LO64,                                 \
-                            lo32 = 1.0 / D - (double)(float)(1.0 / D);                 \
+#define LTNE_INV_SMALL(D, LO)                                  \
+  template <> struct InvSmall<D> {                             \
+    static constexpr double hi = 1.0 / D, lo = LO;             \
   };
 LTNE_INV_SMALL(5, -0x1.999999999999ap-57)
 LTNE_INV_SMALL(6, 0x1.5555555555555p-57)
@@ -121,8 +121,14 @@ LTNE_INV_SMALL(36, 0x1.c71c71c71c71cp-60)
 #undef LTNE_INV_SMALL
 template <int D, typename C>
 LTNE_HD C div_small(C x) {
-  const C xl = x * C(std::is_same<C, double>::value ? InvSmall<D>::lo64 : InvSmall<D>::lo32);
-  return cfma_<C>(x, C(InvSmall<D>::hi), xl);
+  const C hi = C(InvSmall<D>::hi);
+  if constexpr (std::is_same<C, double>::value) {
+    return cfma_<C>(x, hi, x * InvSmall<D>::lo);
+  } else {
+    const C q = x * hi;
+    const C r = cfma_<C>(-C(D), q, x);
+    return cfma_<C>(r, hi, q);
+  }
 }
 
 // Reciprocal and square root of non-conserved quantities (porosity-derived
@@ -309,7 +315,7 @@ LTNE_HD void collide(const NodeParams<C>& P, const Macro<C>& m, C (&f)[9],
   const C ms6 = m6 - P.s_q * (m6 + ruy) - P.half_q * rFy;
   const C ms7 = m7 - P.s_nu * (m7 - meq7) + P.half_nu * S7;
   const C ms8 = m8 - P.s_nu * (m8 - meq8) + P.half_nu * S8;
-  // df* = M^-1 m* (the factors 1/4 and 1/2 are exact and ride on the sums' FMAs)
+  // df* = M^-1 m*
   const C r0 = div_small<9, C>(ms0);
   const C r1 = div_small<36, C>(ms1);
   const C r2 = div_small<36, C>(ms2);
@@ -317,19 +323,20 @@ LTNE_HD void collide(const NodeParams<C>& P, const Macro<C>& m, C (&f)[9],
   const C r4 = div_small<12, C>(ms4);
   const C r5 = div_small<6, C>(ms5);
   const C r6 = div_small<12, C>(ms6);
+  const C r7 = ms7 * C(0.25), r8 = ms8 * C(0.25);
   const C ax = r0 - r1 - C(2) * r2;  // common part of i = 1..4
   const C dg = r0 + C(2) * r1 + r2;  // common part of i = 5..8
   const C px = r3 - C(2) * r4, py = r5 - C(2) * r6;
   const C qx = r3 + r4, qy = r5 + r6;
   f[0] = r0 - C(4) * r1 + C(4) * r2;
-  f[1] = ax + px + ms7 * C(0.25);
-  f[2] = ax + py - ms7 * C(0.25);
-  f[3] = ax - px + ms7 * C(0.25);
-  f[4] = ax - py - ms7 * C(0.25);
-  f[5] = dg + qx + qy + ms8 * C(0.25);
-  f[6] = dg - qx + qy - ms8 * C(0.25);
-  f[7] = dg - qx - qy + ms8 * C(0.25);
-  f[8] = dg + qx - qy - ms8 * C(0.25);
+  f[1] = ax + px + r7;
+  f[2] = ax + py - r7;
+  f[3] = ax - px + r7;
+  f[4] = ax - py - r7;
+  f[5] = dg + qx + qy + r8;
+  f[6] = dg - qx + qy - r8;
+  f[7] = dg - qx - qy + r8;
+  f[8] = dg + qx - qy - r8;
 
   // ---- temperatures
   const C Srf = m.Srf, Srs = m.Srs;  // Eq. 42
@@ -350,13 +357,13 @@ LTNE_HD void collide(const NodeParams<C>& P, const Macro<C>& m, C (&f)[9],
     }
     const C ns3 = n3 - P.zeta_e * (n3 - P.c3 * m.dTf) + P.c3_f * Srf;
     const C ns4 = n4 - P.zeta_nu * n4;
-    const C t0 = div_small<5, C>(ns0);
-    const C t3 = div_small<20, C>(ns3);
+    const C t0 = div_small<5, C>(ns0), t1 = ns1 * C(0.5), t2 = ns2 * C(0.5);
+    const C t3 = div_small<20, C>(ns3), t4 = ns4 * C(0.25);
     gf[0] = t0 - C(4) * t3;
-    gf[1] = t0 + ns1 * C(0.5) + t3 + ns4 * C(0.25);
-    gf[2] = t0 + ns2 * C(0.5) + t3 - ns4 * C(0.25);
-    gf[3] = t0 - ns1 * C(0.5) + t3 + ns4 * C(0.25);
-    gf[4] = t0 - ns2 * C(0.5) + t3 - ns4 * C(0.25);
+    gf[1] = t0 + t1 + t3 + t4;
+    gf[2] = t0 + t2 + t3 - t4;
+    gf[3] = t0 - t1 + t3 + t4;
+    gf[4] = t0 - t2 + t3 - t4;
   }
   {
     const C n1 = gs[1] - gs[3], n2 = gs[2] - gs[4];
@@ -367,13 +374,13 @@ LTNE_HD void collide(const NodeParams<C>& P, const Macro<C>& m, C (&f)[9],
     const C ns2 = n2 - P.eta_a * n2;
     const C ns3 = n3 - P.eta_e * (n3 - P.c3 * m.dTs) + P.c3_s * Srs;
     const C ns4 = n4 - P.eta_nu * n4;
-    const C t0 = div_small<5, C>(ns0);
-    const C t3 = div_small<20, C>(ns3);
+    const C t0 = div_small<5, C>(ns0), t1 = ns1 * C(0.5), t2 = ns2 * C(0.5);
+    const C t3 = div_small<20, C>(ns3), t4 = ns4 * C(0.25);
     gs[0] = t0 - C(4) * t3;
-    gs[1] = t0 + ns1 * C(0.5) + t3 + ns4 * C(0.25);
-    gs[2] = t0 + ns2 * C(0.5) + t3 - ns4 * C(0.25);
-    gs[3] = t0 - ns1 * C(0.5) + t3 + ns4 * C(0.25);
-    gs[4] = t0 - ns2 * C(0.5) + t3 - ns4 * C(0.25);
+    gs[1] = t0 + t1 + t3 + t4;
+    gs[2] = t0 + t2 + t3 - t4;
+    gs[3] = t0 - t1 + t3 + t4;
+    gs[4] = t0 - t2 + t3 - t4;
   }
 }
 
