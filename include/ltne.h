@@ -249,7 +249,9 @@ int64_t ltne_kernel_launch_count(const ltne_handle* h);
    (16-bit storage) advance two steps per launch, in strips that do not
    depend on the block shape; with one (cavity walls, FP32, FP16 or BF16
    storage), lattices up to about 200 x 200 advance up to four, in tiles.  The
-   results are the same bits.  May be called at any time between steps.
+   results are the same bits.  FP64 cavities at the default shape step from a
+   list of nodes in one-warp blocks, again the same bits.  May be called at any
+   time between steps.
    LTNE_ERR_INVALID_ARG for other schedules. */
 int ltne_set_schedule(ltne_handle* h, int32_t block_x, int32_t block_y,
                       int32_t nodes_per_thread);

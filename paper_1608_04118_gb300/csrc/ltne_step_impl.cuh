@@ -269,6 +269,47 @@ __global__ void __launch_bounds__(256) k_step(const S* __restrict__ src, S* __re
                       write_macros, tick, nullptr, um_in, um_out, slab_walls);
 }
 
+// One step of a cavity from a list of its nodes in blocks of one warp: the
+// wall nodes first (left and right column, bottom and top row without the
+// corners), then from a whole warp on the interior.  For FP64, which is bound
+// by the FP64 pipe (two lanes per SM, 16 cycles per warp and operation): a
+// wall node in a warp makes the whole warp pay for its rebuild, which is 60 %
+// more operations and hits every warp of a 64-wide row, and one-warp blocks
+// spread a small lattice over all SMs.  us a step, 64 x 2 blocks -> list:
+// 301 x 211 60.0 -> 43.1, 600 x 500 220 -> 177, 1024^2 688 -> 599, 64^2 19.4 -> 17.6
+// (there one wall warp's chain of dependent FP64 operations, 15 us, is the bound;
+// half-filled warps take as long as full ones).
+template <typename S, typename C>
+__global__ void __launch_bounds__(32) k_step_list(
+    const S* __restrict__ src, S* __restrict__ dst, const C* __restrict__ phi_field,
+    C* __restrict__ mac, const NodeParams<C> P, const int nx, const int ny, const int64_t pitch,
+    const int64_t plane, const C scale, const C inv_scale, const int write_macros,
+    const C* __restrict__ um_in, C* __restrict__ um_out) {
+  grid_dep_wait();
+  const int walls = 2 * ny + 2 * (nx - 2), first = (walls + 31) & ~31;
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  int x, y;
+  if (i < first) {
+    if (i >= walls) return;
+    if (i < 2 * ny) {
+      x = i < ny ? 0 : nx - 1;
+      y = i < ny ? i : i - ny;
+    } else {
+      const int k = i - 2 * ny;
+      y = k < nx - 2 ? 0 : ny - 1;
+      x = 1 + (k < nx - 2 ? k : k - (nx - 2));
+    }
+  } else {
+    const int k = i - first, w = nx - 2;
+    if (k >= w * (ny - 2)) return;
+    y = k / w;
+    x = 1 + k - y * w;
+    ++y;
+  }
+  step_node<S, C, BC_CAVITY>(src, dst, phi_field, mac, P, x, y, nx, ny, pitch, plane, scale,
+                             inv_scale, write_macros, 0u, nullptr, um_in, um_out);
+}
+
 // S_0 from the fields held in the macro planes (rho, ux, uy, Tf, Ts), then
 // its macroscopic values (overwriting the planes) and its collision.
 template <typename S, typename C>
@@ -322,6 +363,15 @@ cudaError_t launch_step_t(const LatticeArgs& a, const NodeParams<double>& Pd, St
   const bool ch = a.chained != 0;
   const dim3 g = grid, b = block;
   cudaError_t e;
+  if constexpr (sizeof(C) == 8) {  // the default schedule of FP64 cavities (64 x 2)
+    if (a.bc == BC_CAVITY && s.bx == 64 && s.by == 2) {
+      const int64_t walls = 2 * (int64_t)a.ny + 2 * (a.nx - 2);
+      const int64_t nodes = (walls + 31) / 32 * 32 + (int64_t)(a.nx - 2) * (a.ny - 2);
+      return launch_kernel(ch, k_step_list<S, C>, dim3((unsigned)((nodes + 31) / 32)), dim3(32), 0,
+                           st, src, dst, phi, mac, P, a.nx, a.ny, a.pitch, a.plane, scale,
+                           inv_scale, a.write_macros, um_in, um_out);
+    }
+  }
 #define LTNE_STEP_LAUNCH(bc, walls)                                                            \
   e = launch_kernel(ch, k_step<S, C, bc>, g, b, 0, st, src, dst, phi, mac, P, a.nx, a.ny,       \
                     a.pitch, a.plane, scale, inv_scale, a.write_macros, a.tick_in, a.tick_out,  \
