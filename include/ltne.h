@@ -248,8 +248,8 @@ int64_t ltne_kernel_launch_count(const ltne_handle* h);
    walls and no local h_v, lattices of 2^22 nodes or more (FP32) or 2^24
    (16-bit storage) advance two steps per launch, in strips that do not
    depend on the block shape; with one (cavity walls, FP32, FP16 or BF16
-   storage), lattices up to about 200 x 200 advance up to four, in tiles.  The
-   results are the same bits.  FP64 cavities at the default shape step from a
+   storage), lattices up to about 200 x 200 advance up to four, in tiles, and
+   FP32 lattices of 2^20 nodes or more without local h_v two.  The results are the same bits.  FP64 cavities at the default shape step from a
    list of nodes in one-warp blocks, again the same bits.  May be called at any
    time between steps.
    LTNE_ERR_INVALID_ARG for other schedules. */

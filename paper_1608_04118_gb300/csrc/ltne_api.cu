@@ -532,18 +532,21 @@ LatticeArgs lattice_args(const ltne_handle* h, int src_buf, int write_macros) {
 // thread: two where k_step2_pair (ltne_march.cuh) is the faster form.  Its
 // strips and segments need enough rows of waves to fill the GPU: FP32 from
 // 2^22 nodes (2048^2 96 -> 84 us a step; 1024^2 27 -> 30), 16-bit storage from
-// 2^24 (4096^2 FP16 303 -> 288; 2048^2 81 -> 90).  One node per thread, FP32
+// 2^24 (4096^2 FP16 307 -> 296; 2048^2 82 -> 92).  One node per thread, FP32
 // arithmetic: four where one block per SM holds the lattice in tiles of
 // k_step_tile (ltne_tile.cuh; up to about 200 x 200: 192^2 2.37 -> 2.18; with
-// two blocks per SM 256^2 2.88 -> 2.95).
+// two blocks per SM 256^2 2.88 -> 2.95); two by k_step2_node for FP32 from 2^20
+// (1024^2 25.7 -> 24.3, 1448^2 50 -> 43; 724^2 10.9 -> 13.6; the 16-bit forms are
+// bound by issue already).
 int steps_per_launch(const ltne_handle* h) {
   const ltne_params& p = h->p;
   if (h->slab || h->shape.tma || p.bc != LTNE_BC_CAVITY || p.storage == LTNE_F64) return 1;
+  const int64_t nodes = (int64_t)p.nx * p.ny;
   if (h->shape.pair) {
-    const int64_t nodes = (int64_t)p.nx * p.ny;
     return !p.hv_local && nodes >= (int64_t)1 << (p.storage == LTNE_F32 ? 22 : 24) ? 2 : 1;
   }
-  return h->shape.tiles.ntx ? kTileSteps : 1;
+  if (h->shape.tiles.ntx) return kTileSteps;
+  return p.storage == LTNE_F32 && !p.hv_local && nodes >= (int64_t)1 << 20 ? 2 : 1;
 }
 
 cudaError_t launch_step(ltne_handle* h, int src_buf, int write_macros, cudaStream_t st,

@@ -20,11 +20,11 @@
 // FMA pipe (busy 69 % of the cycles at 4096^2: a paired instruction holds it
 // for two), with 63 % of the issue slots taken; FP32, that and the rows' loads
 // (DRAM at 70 % of the copy).  Measured, us a step, one-step kernel -> this:
-//   4096^2 FP32, per-node porosity   374 -> 275  (61.1 GLUPS)
+//   4096^2 FP32, per-node porosity   374 -> 278  (60.2 GLUPS)
 //   2048^2 FP32, per-node porosity    96 -> 84
-//   8192^2 FP16, uniform porosity    993 -> 930  (72.2 GLUPS)
-//   8192^2 FP16, per-node porosity  1193 -> 1034
-//   8192^2 BF16, per-node porosity  1132 -> 949
+//   8192^2 FP16, uniform porosity   1003 -> 964  (69.6 GLUPS)
+//   8192^2 FP16, per-node porosity  1205 -> 1068
+//   8192^2 BF16, per-node porosity  1132 -> 987
 // One warp per block: blocks of four warps keep the slots of finished warps
 // (4096^2: 287).  20 blocks per SM, 96 registers: at 80 registers and 24
 // blocks the spills cost more than the warps give (348).  The next row's
@@ -340,8 +340,8 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
 // Rows per segment.  A segment of s rows costs 2 s + 2 row steps, its first
 // row of waves fills up and its last drains in about 0.7 of a segment's
 // time (fitted to sweeps of s: 6, 10, 14, 20 took 84, 88, 91, 106 us a step at
-// 2048^2 FP32, 284, 277, 279, 285 at 4096^2 FP32, and 10, 14, 20, 24 took 984,
-// 962, 951, 949 at 8192^2 BF16).  Not above 24: the rows in work at one time
+// 2048^2 FP32, 284, 277, 279, 285 at 4096^2 FP32, and 10, 14, 20, 24 took 1018,
+// 996, 984, 982 at 8192^2 BF16).  Not above 24: the rows in work at one time
 // then spread over more memory than L2 and the address translation hold
 // (4096^2: 404 us with one wave of 98-row segments).
 inline int march_rows(int strips, int ny, int warps) {
@@ -373,6 +373,104 @@ cudaError_t launch_step2_pair_t(const LatticeArgs& a, const NodeParams<double>& 
                        static_cast<const float*>(a.phi), static_cast<float*>(a.mac), P, P1, a.nx,
                        a.ny, (uint32_t)a.pitch, (uint32_t)a.plane, a.enc_scale,
                        1.0f / a.enc_scale, a.write_macros, a.tick_in, a.tick_out, seg);
+}
+
+// The same walk with one node per lane (FP32 storage), for lattices whose
+// schedule has one node per thread: strips of 32 nodes, 30 of which take the
+// second step, and segments of 8 rows (4, 6, 8, 12, 16 rows took 24.3, 24.9, 24.3,
+// 24.6, 28.1 us a step at 1024^2, 82, 79, 78, 79, 79 at 2048 x 2047).  64 registers,
+// 32 one-warp blocks per SM.  Bound: instruction issue, and at 1024^2 the last
+// wave of segments.  Measured, us a step, one-step kernel -> this: 1024^2 FP32,
+// per-node porosity, 25.7 -> 24.3, 1448^2 50.2 -> 42.7, 2048 x 2047 96.2 -> 78.2 (724^2
+// 10.9 -> 13.6: too few segments).  The bits of two launches of k_step.
+constexpr int kMarchNodes = 30;
+constexpr int kMarchNodeBlocks = 32;
+constexpr int kMarchNodeRows = 8;
+
+static __global__ void __launch_bounds__(32, kMarchNodeBlocks) k_step2_node(
+    const float* __restrict__ src, float* __restrict__ dst, const float* __restrict__ phi,
+    float* __restrict__ mac, const __grid_constant__ NodeParams<float> P, const int nx,
+    const int ny, const int64_t pitch, const int64_t plane, const int write_macros,
+    const int seg_rows) {
+  __shared__ float line[19][32];  // the slots of k_step2_pair
+  grid_dep_wait();
+  const int lane = threadIdx.x;
+  int x = blockIdx.x * kMarchNodes + lane;
+  const bool own = x < nx && (lane > 0 || x == 0) && (lane < 31 || x == nx - 1);
+  x = min(x, nx - 1);
+  const int side = x == 0 ? 0 : (x == nx - 1 ? 1 : -1);
+  const int cx = min(max(x, 1), nx - 2);
+  const bool side_strip = __any_sync(0xffffffffu, side >= 0);
+  // a side node's rebuild takes the values of the node it is rebuilt from
+  const int from = side == 0 ? lane + 1 : (side == 1 ? lane - 1 : lane);
+  const int ya = blockIdx.y * seg_rows, yb = min(ny, ya + seg_rows);
+  const int r0 = max(ya - 1, 0), r1 = min(yb, ny - 1);
+  const uint32_t pi = (uint32_t)pitch;
+  for (int r = r0; r <= r1; ++r) {
+    const int j = r - 1;
+    const bool wall_next = j == 1 || j == ny - 2;
+    int y = r, cy = r == 0 ? 1 : (r == ny - 1 ? ny - 2 : r);
+    float f[9], gf[5], gs[5], t[19];
+    Pops<float, float>::pull(src, pitch, plane, cx, cx - 1, cx + 1, cy, cy - 1, cy + 1, 1.0f, f, gf,
+                             gs);
+    auto value = [&](int i) -> float& {
+      return i < 9 ? f[i < 9 ? i : 0] : (i < 14 ? gf[(i - 9) % 5] : gs[(i - 9) % 5]);
+    };
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+      const uint32_t off = (uint32_t)y * pi + x, noff = (uint32_t)cy * pi + cx;
+      Macro<float> m;
+      update_node<float, BC_CAVITY>(P, phi, off, noff, side >= 0 ? side : (y != cy ? 2 : -1),
+                                    nullptr, nullptr, plane, nullptr, f, gf, gs, m);
+      if (pass == 0) {
+        const int par = r & 1;
+#pragma unroll
+        for (int i = 0; i < 19; ++i) {
+          float& v = value(i);
+          if (value_ex(i) > 0) v = __shfl_up_sync(0xffffffffu, v, 1);
+          if (value_ex(i) < 0) v = __shfl_down_sync(0xffffffffu, v, 1);
+          if (value_ey(i) >= 0) {
+            constexpr int slot[19] = {0, 1, 9, 2, 0, 10, 11, 0, 0, 3, 4, 12, 5, 0, 6, 7, 13, 8, 0};
+            float& s = line[value_ey(i) > 0 && par ? slot[i] + 5 : slot[i]][lane];
+            const float o = s;
+            s = v;
+            v = o;
+          }
+        }
+        if (r < r0 + 2) break;  // the line is not full yet
+        if (side_strip) {
+#pragma unroll
+          for (int i = 0; i < 19; ++i) value(i) = __shfl_sync(0xffffffffu, value(i), from);
+        }
+        if (wall_next) {
+#pragma unroll
+          for (int i = 0; i < 19; ++i) t[i] = value(i);
+        }
+        y = cy = j;
+        continue;
+      }
+      if (own) {
+        if (write_macros) store_macros<float>(mac, plane, off, m);
+        Pops<float, float>::store(dst, plane, off, 1.0f, f, gf, gs, 0u, 0u);
+      }
+      if (!wall_next || pass == 2) break;
+      y = j == 1 ? 0 : ny - 1;
+#pragma unroll
+      for (int i = 0; i < 19; ++i) value(i) = t[i];
+    }
+  }
+}
+
+inline cudaError_t launch_step2_node(const LatticeArgs& a, const NodeParams<double>& Pd,
+                                     cudaStream_t st) {
+  const int strips = a.nx <= 32 ? 1 : (a.nx - 32 + kMarchNodes - 1) / kMarchNodes + 1;
+  const dim3 grid(strips, (a.ny + kMarchNodeRows - 1) / kMarchNodeRows);
+  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  return launch_kernel(a.chained != 0, k_step2_node, grid, dim3(32), 0, st,
+                       static_cast<const float*>(a.src), static_cast<float*>(a.dst),
+                       static_cast<const float*>(a.phi), static_cast<float*>(a.mac),
+                       cast_params<float>(Pd), a.nx, a.ny, a.pitch, a.plane, a.write_macros,
+                       kMarchNodeRows);
 }
 
 }  // namespace ltne

@@ -334,6 +334,9 @@ cudaError_t launch_step_tma_t(const LatticeArgs& a, const NodeParams<double>& Pd
   namespace ltne {                                                                             \
   cudaError_t launch_step_##tag(const LatticeArgs& a, const NodeParams<double>& P,             \
                                 StepShape s, cudaStream_t st) {                                \
+    if constexpr (std::is_same<S, float>::value) {                                             \
+      if (s.steps == 2 && !s.pair && !s.tiles.ntx) return launch_step2_node(a, P, st);         \
+    }                                                                                          \
     if (s.steps > 1)                                                                           \
       return s.pair ? launch_step2_pair_t<S>(a, P, st)                                         \
                     : launch_step_tile_t<S, float>(a, P, s, st);                               \

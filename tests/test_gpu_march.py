@@ -1,4 +1,5 @@
-"""Two time steps per launch (k_step2_pair) against one step at a time.
+"""Two time steps per launch (k_step2_pair, k_step2_node) against one step at
+a time.
 
 Large cavities with two nodes per thread advance two steps in one pass; the
 fields, the populations and the observables have to be the bits of single
@@ -20,8 +21,8 @@ torch = pytest.importorskip("torch")
 NODES = {"f32": 1 << 22, "f16": 1 << 24, "bf16": 1 << 24}
 
 
-def _run(cfg, storage, phi, fields, chunks):
-    c = cavity_for(cfg, storage=storage, phi=phi).set_schedule(32, 4, 2)
+def _run(cfg, storage, phi, fields, chunks, schedule=(32, 4, 2)):
+    c = cavity_for(cfg, storage=storage, phi=phi).set_schedule(*schedule)
     c.set_fields(porosity=phi, **fields)
     for n in chunks:
         c.step(n)
@@ -49,8 +50,28 @@ def test_two_steps_per_launch_give_the_bits_of_single_steps(storage, nx, ny, ste
     cfg = dict(W.random_params(301, nx, ny), thermal_correction=correction, ergun=bool(field))
     fields = W.random_fields(nx, ny, 302)
     phi = W.porosity_field(nx, ny, 0.4, 0.9, seed=303).reshape(-1) if field else None
-    a = _run(cfg, storage, phi, fields, [steps])
-    b = _run(cfg, storage, phi, fields, [1] * steps)
+    _same(_run(cfg, storage, phi, fields, [steps]), _run(cfg, storage, phi, fields, [1] * steps),
+          steps)
+
+
+@pytest.mark.parametrize("nx,ny,steps,field,correction", [
+    (31, 34_000, 5, True, 0), (32, 33_000, 4, False, 0), (33, 32_000, 5, True, 1),
+    (60, 17_600, 4, True, 0), (61, 17_300, 5, False, 0), (62, 17_001, 4, True, 0),
+    (63, 16_900, 3, True, 0), (262_144, 4, 5, True, 0), (209_716, 5, 4, True, 0),
+    (1027, 1025, 75, True, 0)])
+def test_two_steps_with_one_node_per_thread(nx, ny, steps, field, correction):
+    """The one-node walk: widths around one and two strips of 30 nodes."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    assert nx * ny >= 1 << 20
+    cfg = dict(W.random_params(311, nx, ny), thermal_correction=correction, ergun=bool(field))
+    fields = W.random_fields(nx, ny, 312)
+    phi = W.porosity_field(nx, ny, 0.4, 0.9, seed=313).reshape(-1) if field else None
+    _same(_run(cfg, "f32", phi, fields, [steps], (64, 2, 1)),
+          _run(cfg, "f32", phi, fields, [1] * steps, (64, 2, 1)), steps)
+
+
+def _same(a, b, steps):
     for k in a[0]:
         assert np.array_equal(a[0][k], b[0][k]), k
     assert a[1] == b[1]
