@@ -476,11 +476,12 @@ def form_plain_1024(stream, peak, gpu, steps=2000, warmup=500):
     rate = n * n * steps / t / 1e6
     sched = list(cav.schedule)
     cav.close()
-    achieved = BYTES_PER_LUP["f32"] * rate * 1e6 / 1e9
+    bytes_per_lup = BYTES_PER_LUP["f32"] * launches / steps  # a launch may advance two steps
+    achieved = bytes_per_lup * rate * 1e6 / 1e9
     return {"mlups": rate, "lattice": "%dx%d" % (n, n), "steps": steps, "warmup": warmup,
             "schedule": sched, "gpu_launches": launches,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "bytes_per_lup": BYTES_PER_LUP["f32"]},
+                         "frac": achieved / peak, "bytes_per_lup": bytes_per_lup},
             "clocks": clocks}
 
 

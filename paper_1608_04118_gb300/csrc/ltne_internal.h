@@ -47,8 +47,9 @@ struct LatticeArgs {
 // on the stream exit, before that grid's completion is signalled, and waits
 // here for the completion (and its memory flush) before touching global
 // memory; without the launch attribute the wait is a no-op.  Every thread
-// of a kernel that may be launched so executes it before any global access
-// or early return, so each grid completes only after its predecessor did.
+// of a kernel that may be launched so executes it before its early return and
+// before it touches anything that a kernel it may be chained to writes, so
+// each grid completes only after its predecessor did.
 __device__ __forceinline__ void grid_dep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
