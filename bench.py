@@ -632,10 +632,7 @@ def run_batch(args):
     t_seq = ev0.elapsed_time(ev1) / 1e3
     seq = nodes * k_seq / t_seq / 1e6
     peak, kind = load_peaks()
-    # one pass over the lattice may advance two steps (k_step2_pair): the bytes
-    # a launch has to move, and its time, per launch and per step
-    per_launch = t / launches
-    bytes_per_lup = BYTES_PER_LUP[args.storage] * launches / args.steps
+    per_launch = t / args.steps
     achieved = 152 * nodes / per_launch / 1e9
     line = {"metric": "MLUPS (batched, 256 cavities)", "value": value, "unit": UNIT,
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
