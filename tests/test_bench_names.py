@@ -28,3 +28,7 @@ def unresolved():
 
 def test_the_batch_workload_uses_no_missing_name():
     assert not {n for f, n in unresolved() if f == "run_batch"}
+
+
+def test_no_function_of_the_benchmark_uses_a_missing_name():
+    assert not unresolved()
