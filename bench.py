@@ -136,12 +136,15 @@ def load_peaks():
     return 6800.0, "fallback"
 
 
-def kernel_traffic(storage, n, npt):
+def kernel_traffic(storage, n, npt, steps, launches):
     """ncu DRAM bytes per launch of the step kernel (storage type, nodes per
-    thread) from the committed profile summary, if it was taken on the
-    current kernel source: (bytes, how) with how "measured at NxN" when the
-    capture is of this lattice, else "scaled from NxN" (traffic grows with
-    the node count), or (None, reason)."""
+    thread, time steps per launch) from the committed profile summary, if it
+    was taken on the current kernel source: (bytes, how) with how "measured at
+    NxN" when the capture is of this lattice, else "scaled from NxN" (traffic
+    grows with the node count), or (None, reason).  A capture holds for timed
+    launches that all advance as many steps as the captured one."""
+    if steps % launches:
+        return None, "launches of different step counts"
     p = os.path.join(ROOT, "profiles", "step_traffic.json")
     if not os.path.exists(p):
         return None, "no capture"
@@ -152,7 +155,8 @@ def kernel_traffic(storage, n, npt):
 
         if d.get("source_hash") != B.kernel_source_hash():
             return None, "capture predates the current kernel source"
-        cands = [e for k, e in d["entries"].items() if k.startswith("%s/npt%d" % (storage, npt))]
+        form = "%s/npt%d/steps%d/" % (storage, npt, steps // launches)
+        cands = [e for k, e in d["entries"].items() if k.startswith(form)]
         if not cands:
             return None, "no capture of this form"
         exact = [e for e in cands if int(e["nodes"]) == n * n]
@@ -1000,7 +1004,7 @@ def main():
     bytes_per_lup = BYTES_PER_LUP[args.storage] * launches / args.steps
     peak, peak_kind = load_peaks()
     achieved = BYTES_PER_LUP[args.storage] * nodes / per_launch / 1e9
-    traffic, traffic_how = kernel_traffic(args.storage, n, schedule[2])
+    traffic, traffic_how = kernel_traffic(args.storage, n, schedule[2], args.steps, launches)
     ob = cav.observables()
     # The FP64 observables: one ltne_observables call (the reduction pass
     # over the fields and the residual snapshot, its combination, the
