@@ -170,6 +170,19 @@ def kernel_traffic(storage, n, npt, steps, launches):
         return None, "unreadable capture (%s)" % type(ex).__name__
 
 
+def step_kernel(storage, schedule, staged, n, steps, launches):
+    """The kernel that made the timed steps of an n x n cavity with per-node
+    porosity: by the schedule (block_x, block_y, nodes per thread), whether
+    tiles were staged, and whether its launches advanced more than a step."""
+    if launches < steps:  # one node per thread: tiles up to about 200 x 200, the walk from 1024 x 1024
+        return "k_step2_pair" if schedule[2] == 2 else "k_step2_node" if n >= 1024 else "k_step_tile"
+    if staged:
+        return "k_step_tma"
+    if storage == "f64" and tuple(schedule[:2]) == (64, 2):
+        return "k_step_list"
+    return "k_step_pair" if schedule[2] == 2 else "k_step"
+
+
 class ClockSampler:
     FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
               "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -968,7 +981,7 @@ def main():
         cav.set_schedule(bx, by, args.npt or cav.schedule[2])
     if args.staging >= 0:
         cav.set_staging(args.staging)
-    schedule = cav.schedule
+    schedule, staged = cav.schedule, cav.staging
     cav.set_fields(porosity=phi)
 
     def barrier():
@@ -998,8 +1011,9 @@ def main():
     t_max = max_over_ranks(t, dev)
     nodes = n * n
     value = whole_job_mlups(nodes, args.steps, ws, t_max)
-    # one pass over the lattice may advance two steps (k_step2_pair): the bytes
-    # a launch has to move, and its time, per launch and per step
+    kernel = step_kernel(args.storage, schedule, staged, n, args.steps, launches)
+    # one pass over the lattice may advance several steps: the bytes a launch
+    # has to move, and its time, per launch and per step
     per_launch = t / launches
     bytes_per_lup = BYTES_PER_LUP[args.storage] * launches / args.steps
     peak, peak_kind = load_peaks()
@@ -1107,9 +1121,7 @@ def main():
                      # the ncu-counted bytes of one launch over the launch time
                      "achieved_dram": None if traffic is None else traffic / per_launch / 1e9,
                      "kernel": "%s<%s> (%d launches for %d steps of %d nodes)"
-                               % ("k_step2_pair" if launches < args.steps else
-                                  "k_step_pair" if schedule[2] == 2 else "k_step", args.storage,
-                                  launches, args.steps, nodes)},
+                               % (kernel, args.storage, launches, args.steps, nodes)},
         "observables_reduction": {"ms": obs_s * 1e3,
                                   "note": "one ltne_observables call after a one-step call: "
                                           "both passes, the read-back and its synchronisation",
