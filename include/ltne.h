@@ -182,7 +182,8 @@ int ltne_set_fields(ltne_handle* h, const double* porosity, const double* rho,
 
 /* Advance n >= 0 time steps (collision, streaming and walls per step),
    asynchronously on the handle's stream, replaying a cached CUDA graph of
-   steps where it can. */
+   steps where it can.  LTNE_ERR_CUDA, with no step made, for a lattice of more
+   than 65535 block_y rows (see ltne_set_schedule). */
 int ltne_step(ltne_handle* h, int64_t n);
 
 /* Reduce the current fields to *out (synchronises the stream).  Returns

@@ -1039,6 +1039,12 @@ int ltne_step(ltne_handle* h, int64_t n) {
   if (!h || n < 0 || h->slab) return LTNE_ERR_INVALID_ARG;
   if (!h->ws || !h->fields_set) return LTNE_ERR_STATE;
   if (n == 0) return LTNE_OK;
+  // A one-step launch has a block row per block_y rows of the lattice.  Where
+  // that is more than a grid holds the call fails before its first step, also
+  // if kernels of several steps (whose grids are smaller) could make a part of
+  // them: whether a call is accepted does not depend on n.
+  if (!h->shape.tma && (h->p.ny - 1) / h->shape.by >= kMaxGridY)
+    return fail_cuda(cudaErrorInvalidConfiguration);
   int64_t plain = n - 1;  // the last step also writes the macroscopic fields
   cudaError_t e;
   // the lattice constants are arguments of the captured launches: a graph

@@ -82,6 +82,7 @@ cudaError_t launch_kernel(bool chained, void (*k)(KArgs...), dim3 grid, dim3 blo
 // each advancing one node or (pair = 1, FP32 arithmetic only, at most
 // kPairBlockThreads threads per block) two neighbouring nodes of a row.
 constexpr int kSMs = 152;  // streaming multiprocessors of a GB300
+constexpr int kMaxGridY = 65535;  // blocks of a grid in y
 constexpr int kPairBlockThreads = 128;
 // Tiles of k_step_tile (plan_tiles); ntx = 0: the lattice is too large for it.
 struct TilePlan {

@@ -367,7 +367,7 @@ cudaError_t launch_step2_pair_t(const LatticeArgs& a, const NodeParams<double>& 
   const int strips = npairs <= 32 ? 1 : (npairs - 32 + kMarchPairs - 1) / kMarchPairs + 1;
   const int seg = march_rows(strips, a.ny, kSMs * kMarchBlocks);
   const dim3 grid(strips, (a.ny + seg - 1) / seg);
-  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  if (grid.y > (unsigned)kMaxGridY) return cudaErrorInvalidValue;
   return launch_kernel(a.chained != 0, a.nx % 2 ? k_step2_pair<S, true> : k_step2_pair<S, false>,
                        grid, dim3(32), 0, st, static_cast<const S*>(a.src), static_cast<S*>(a.dst),
                        static_cast<const float*>(a.phi), static_cast<float*>(a.mac), P, P1, a.nx,
@@ -465,7 +465,7 @@ inline cudaError_t launch_step2_node(const LatticeArgs& a, const NodeParams<doub
                                      cudaStream_t st) {
   const int strips = a.nx <= 32 ? 1 : (a.nx - 32 + kMarchNodes - 1) / kMarchNodes + 1;
   const dim3 grid(strips, (a.ny + kMarchNodeRows - 1) / kMarchNodeRows);
-  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  if (grid.y > (unsigned)kMaxGridY) return cudaErrorInvalidValue;
   return launch_kernel(a.chained != 0, k_step2_node, grid, dim3(32), 0, st,
                        static_cast<const float*>(a.src), static_cast<float*>(a.dst),
                        static_cast<const float*>(a.phi), static_cast<float*>(a.mac),
