@@ -1131,12 +1131,19 @@ int ltne_get_fields(ltne_handle* h, double* rho, double* ux, double* uy, double*
     const cudaError_t es = cudaStreamSynchronize(h->stream);
     return fail_cuda(e != cudaSuccess ? e : es);
   }
-  // small lattices: all five planes in one copy, then converted row by row
-  const size_t all = 5 * (size_t)h->plane * h->ec;
+  // small lattices: the planes that are asked for, neighbouring ones in one
+  // copy, then converted row by row
+  const size_t pb = (size_t)h->plane * h->ec, all = 5 * pb;
   if (all <= kPinBytes) {
     cudaError_t e = ensure_pinned(h, all);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(h->pin[0], mac_cur(h), all, cudaMemcpyDeviceToHost, h->stream);
+    for (int k = 0; k < 5 && e == cudaSuccess; ++k) {
+      int run = 0;
+      while (k + run < 5 && dst[k + run]) ++run;
+      if (run)
+        e = cudaMemcpyAsync(h->pin[0] + k * pb, mac_cur(h) + k * pb, run * pb,
+                            cudaMemcpyDeviceToHost, h->stream);
+      k += run;  // the plane after a run was not asked for
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return fail_cuda(e);
     for (int k = 0; k < 5; ++k) {
@@ -1153,7 +1160,7 @@ int ltne_get_fields(ltne_handle* h, double* rho, double* ux, double* uy, double*
             },
             (((int64_t)1 << 18) + nx - 1) / nx);
       };
-      const char* plane = h->pin[0] + (size_t)k * h->plane * h->ec;
+      const char* plane = h->pin[0] + k * pb;
       if (h->ec == 8) convert(reinterpret_cast<const double*>(plane));
       else convert(reinterpret_cast<const float*>(plane));
     }
