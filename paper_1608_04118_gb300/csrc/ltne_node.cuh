@@ -154,7 +154,8 @@ template <typename C> LTNE_HD C sqrt_(C x);
 template <> LTNE_HD double sqrt_<double>(double x) { return sqrt(x); }
 template <> LTNE_HD float sqrt_<float>(float x) {
 #ifdef __CUDA_ARCH__
-  // a subnormal x (a speed below 1e-19) counts as 0
+  // a subnormal x (a speed below 1e-19) counts as 0: beside l0 >= 1/2 and c0
+  // such a speed is far below the last place; where it counts: full_speed
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return x >= 1.17549435e-38f ? x * r : 0.0f;
@@ -166,6 +167,16 @@ template <> LTNE_HD float sqrt_<float>(float x) {
 template <typename C> LTNE_HD C csqrt_(C x);
 template <> LTNE_HD float csqrt_<float>(float x) { return sqrtf(x); }
 template <> LTNE_HD double csqrt_<double>(double x) { return sqrt(x); }
+
+// |u| over FP32's whole range, given the value mag that sqrt_ makes of its
+// square, which is 0 where the square is below the normal range: what Eq. 52
+// takes, whose power 0.644 makes 1e-13 of a speed of 1e-20.
+template <typename C> LTNE_HD C full_speed(C mag, C, C) { return mag; }
+template <> LTNE_HD float full_speed<float>(float mag, float ux, float uy) {
+  if (mag != 0.0f || (ux == 0.0f && uy == 0.0f)) return mag;
+  const float x = 0x1p100f * ux, y = 0x1p100f * uy;  // both below 2^-62 before
+  return 0x1p-100f * sqrt_<float>(x * x + y * y);
+}
 
 // The coefficients at porosity phi (per-node porosity fields).
 //   Darcy K, constant F : c0 = nu_over_K, c1 = Fconst * inv_sqrtK

@@ -86,6 +86,11 @@ template <> LTNE_HD F2 rcp_<F2>(F2 x) { return F2(rcp_<float>(x.v.x), rcp_<float
 template <> LTNE_HD F2 sqrt_<F2>(F2 x) { return F2(sqrt_<float>(x.v.x), sqrt_<float>(x.v.y)); }
 template <> LTNE_HD F2 csqrt_<F2>(F2 x) { return F2(csqrt_<float>(x.v.x), csqrt_<float>(x.v.y)); }
 
+template <> LTNE_HD F2 full_speed<F2>(F2 mag, F2 ux, F2 uy) {
+  return F2(full_speed<float>(mag.v.x, ux.v.x, uy.v.x),
+            full_speed<float>(mag.v.y, ux.v.y, uy.v.y));
+}
+
 // Eq. 52 per lane.
 template <> LTNE_HD F2 hv_local_at<F2>(const NodeParams<F2>& P, F2 um) {
   NodeParams<float> q;
@@ -240,7 +245,7 @@ __device__ __forceinline__ void finish_pair(S* __restrict__ dst,
   if (P.hv_local) set_exchange<F2>(md, hv_local_at<F2>(P, ld_f2(um_in + off)));
   Macro<F2> m;
   macros<F2>(P, md, f, gf, gs, m);
-  if (P.hv_local) st_f2(um_out + off, m.umag);
+  if (P.hv_local) st_f2(um_out + off, full_speed<F2>(m.umag, m.ux, m.uy));
   if (write_macros) {
     st_f2(mac + off, m.drho);
     st_f2(mac + pl + off, m.ux);

@@ -226,7 +226,8 @@ __device__ __forceinline__ void step_node(const S* __restrict__ src, S* __restri
   Macro<C> m;
   update_node<C, BC>(P, phi_field, off, noff, kind, um_in + off, um_in + noff, plane, pre_out, f,
                      gf, gs, m);
-  if (P.hv_local) um_out[off] = m.umag;  // u_m of Eq. 52 for the next state
+  // u_m of Eq. 52 for the next state
+  if (P.hv_local) um_out[off] = full_speed<C>(m.umag, m.ux, m.uy);
   if (write_macros) store_macros<C>(mac, plane, off, m);
   Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, (uint32_t)off, tick);
 }
@@ -326,7 +327,8 @@ __global__ void __launch_bounds__(256) k_init(S* __restrict__ dst,
   Medium<C> md = phi_field ? medium_at<C>(P, phi_field[off]) : P.um;
   if (P.hv_local) {  // u_m of S_0: the initial field's |u|
     const C ux = mac[plane + off], uy = mac[2 * plane + off];
-    set_exchange<C>(md, hv_local_at<C>(P, sqrt_<C>(ux * ux + uy * uy)));
+    set_exchange<C>(
+        md, hv_local_at<C>(P, full_speed<C>(sqrt_<C>(ux * ux + uy * uy), ux, uy)));
   }
   C f[9], gf[5], gs[5];
   equilibrium<C>(P, md.phi, mac[off], mac[plane + off], mac[2 * plane + off],
@@ -341,7 +343,7 @@ __global__ void __launch_bounds__(256) k_init(S* __restrict__ dst,
   }
   Macro<C> m;
   macros<C>(P, md, f, gf, gs, m);
-  if (P.hv_local) um_out[off] = m.umag;
+  if (P.hv_local) um_out[off] = full_speed<C>(m.umag, m.ux, m.uy);
   store_macros<C>(mac, plane, off, m);
   collide<C>(P, m, f, gf, gs);
   Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, (uint32_t)off, 0xffffffffu);

@@ -93,11 +93,11 @@ __global__ void __launch_bounds__(kTileThreads) k_step_tile(
       Macro<C> m;
       update_node<C, BC_CAVITY>(P, phi, off, noff, kind, um, umn, 0, nullptr, f, gf, gs, m);
       if (e == 0) {
-        if (P.hv_local) um_out[off] = m.umag;
+        if (P.hv_local) um_out[off] = full_speed<C>(m.umag, m.ux, m.uy);
         if (write_macros) store_macros<C>(mac, plane, off, m);
         Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, off, tick + s);
       } else {
-        if (P.hv_local) sm.um[out][q] = m.umag;
+        if (P.hv_local) sm.um[out][q] = full_speed<C>(m.umag, m.ux, m.uy);
         Pops<S, C>::store(&sm.pops[out][0][0], kTileNodes, q, scale, f, gf, gs, off, tick + s);
       }
     }
