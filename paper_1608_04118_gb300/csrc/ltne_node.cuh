@@ -22,8 +22,6 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 // Per-node functions compile for host and device (the host copies serve
 // derivative checks of the reverse-mode functions).
 #define LTNE_HD __host__ __device__ __forceinline__
@@ -98,37 +96,22 @@ template <> LTNE_HD double cfma_<double>(double a, double b, double c) {
   return fma(a, b, c);
 }
 
-// x / D for a small integer D.  FP32: the product with hi = RN(1/D) and one
-// residual correction (r = x - D q is exact in an FMA), which removes the
-// systematic bias that the plain product would add at every step -- in FP32,
-// 6 RN(1/6) = 1 + 3e-8 would grow the momentum by that factor per step.  FP64:
-// the reciprocal as hi + lo, lo = RN(1/D - hi), and x hi + x lo with one fused
-// rounding, an operation less: the quotient to within 2^-53 (1 + 2^-52).  (In
-// FP32 that form gives the same bits for every normal significand, but not
-// below 1e-36, where x lo loses bits; a run from exact rest carries that into
-// the last place of its fields, so FP32 keeps the correction.)
-template <int D> struct InvSmall;
-#define LTNE_INV_SMALL(D, LO)                                  \
-  template <> struct InvSmall<D> {                             \
-    static constexpr double hi = 1.0 / D, lo = LO;             \
-  };
-LTNE_INV_SMALL(5, -0x1.999999999999ap-57)
-LTNE_INV_SMALL(6, 0x1.5555555555555p-57)
-LTNE_INV_SMALL(9, 0x1.c71c71c71c71cp-58)
-LTNE_INV_SMALL(12, 0x1.5555555555555p-58)
-LTNE_INV_SMALL(20, -0x1.999999999999ap-59)
-LTNE_INV_SMALL(36, 0x1.c71c71c71c71cp-60)
-#undef LTNE_INV_SMALL
+// x / D for a small integer D: the product with RN(1/D) and one residual
+// correction (r = x - D q is exact in an FMA), which removes the systematic
+// bias that the plain product would add at every step -- in FP32, 6 RN(1/6) =
+// 1 + 3e-8 would grow the momentum by that factor per step.  Correctly rounded
+// for every normal quotient.  (1/D as hi + lo and x hi + x lo in one fused
+// rounding takes an operation less and gives the same bits while x lo is exact
+// enough, but not for the smallest x, where x lo is subnormal: below 1e-36 in
+// FP32, 3e-306 in FP64.  A run from exact rest passes through those values at
+// the front of what spreads from the walls, and carries the difference into
+// the last place of its fields.)
 template <int D, typename C>
 LTNE_HD C div_small(C x) {
-  const C hi = C(InvSmall<D>::hi);
-  if constexpr (std::is_same<C, double>::value) {
-    return cfma_<C>(x, hi, x * InvSmall<D>::lo);
-  } else {
-    const C q = x * hi;
-    const C r = cfma_<C>(-C(D), q, x);
-    return cfma_<C>(r, hi, q);
-  }
+  const C rc = C(1.0 / D);
+  const C q = x * rc;
+  const C r = cfma_<C>(-C(D), q, x);
+  return cfma_<C>(r, rc, q);
 }
 
 // Reciprocal and square root of non-conserved quantities (porosity-derived

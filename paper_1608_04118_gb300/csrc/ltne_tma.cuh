@@ -30,6 +30,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "ltne_march.cuh"
 #include "ltne_tile.cuh"
