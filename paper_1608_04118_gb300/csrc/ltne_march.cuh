@@ -37,7 +37,8 @@
 // The results are the bits of two launches of k_step_pair: the same per-node
 // functions in the same paired arithmetic, the values between the steps as
 // the populations would have stored them (16-bit storage: rounded with the
-// same random words), the odd last node of a row in the one-node arithmetic.
+// same random words), the odd last node of a row in the one-node arithmetic
+// (MarchOdd).
 #pragma once
 
 #include "ltne_pair.cuh"
@@ -213,6 +214,20 @@ template <> __device__ __forceinline__ float element<float>(uint32_t bits) {
 
 constexpr int kMarchPairs = 30;   // pairs of a strip advanced by both steps (of 32 by the first)
 constexpr int kMarchBlocks = 20;  // one-warp blocks per SM (96 registers)
+constexpr int kMarchRows = 24;    // rows of a segment at most (march_rows)
+
+// The lone last node of an odd row runs in the one-node arithmetic, over which
+// one lane takes a warp as long as all 32 would.  So the rows of a segment are
+// spread over the lanes: the first step of the column's nodes is one pass before
+// the walk (of its results the strip needs the five values with e_x = -1), the
+// second step one pass after it, from the values pulled on the way.  With a pass
+// per row, 513 x 32,804 FP16 took 470 us a step, 2049 x 8288 uniform 309, 129 x
+// 32,713 FP32 188 (one step per launch: 413, 288, 185); this way 353, 282, 154.
+template <bool kOdd> struct MarchOdd {
+  uint32_t left[5][32];             // values 3, 6, 7, 12, 17 after the first step, by row
+  float pulled[kMarchRows + 1][19];  // around the column beside, before the second
+};
+template <> struct MarchOdd<false> {};
 
 template <typename S, bool kOdd>
 __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
@@ -225,6 +240,7 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
   using PT = typename PP::T;
   constexpr bool kRandom = Codec<S, float>::kStochastic;
   __shared__ PT line[19][32];  // slots 0-8: e_y = 0, one row; 9-18: e_y = +1, two rows
+  [[maybe_unused]] __shared__ MarchOdd<kOdd> column;
   grid_dep_wait();
   uint32_t tick = 0;
   if constexpr (kRandom) {
@@ -244,6 +260,23 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
   const bool odd_strip = kOdd && __any_sync(0xffffffffu, last);
   const int ya = blockIdx.y * seg_rows, yb = min(ny, ya + seg_rows);
   const int r0 = max(ya - 1, 0), r1 = min(yb, ny - 1);  // rows of the first step
+  if constexpr (kOdd) {
+    if (odd_strip) {  // first step of the column x = nx - 1, row r0 + lane
+      const int y = min(r0 + lane, r1), cy = min(max(y, 1), ny - 2);
+      float f[9], gf[5], gs[5], v[19], mac5[5];
+      uint32_t e[19];
+      Pops<S, float>::pull(src, pi, pl, nx - 2, nx - 3, nx - 1, cy, cy - 1, cy + 1, inv_scale, f,
+                           gf, gs);
+#pragma unroll
+      for (int i = 0; i < 19; ++i) v[i] = i < 9 ? f[i] : (i < 14 ? gf[i - 9] : gs[i - 14]);
+      march_odd<S>(P1, phi, (uint32_t)y * pi + (nx - 1), (uint32_t)cy * pi + (nx - 2), scale, tick,
+                   v, e, mac5);
+      const int from[5] = {3, 6, 7, 12, 17};
+#pragma unroll
+      for (int k = 0; k < 5; ++k) column.left[k][lane] = e[from[k]];
+      __syncwarp();
+    }
+  }
 
   for (int r = r0; r <= r1; ++r) {
     // pass 0: first step of row r; pass 1: second step of row j = r - 1; pass 2:
@@ -254,8 +287,7 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
     F2 f[9], gf[5], gs[5];
     PairPops<S>::pull(src, pl, pi, (int)x0, (int)x0 - 1, (int)x0 + 2, cy, cy - 1, cy + 1, inv_scale,
                       f, gf, gs);
-    F2 t[19];      // pass 1's pulled values, kept for pass 2
-    float to[19];  // those of the node left of the odd last one
+    F2 t[19];  // pass 1's pulled values, kept for pass 2
 #pragma unroll 1
     for (int pass = 0;; ++pass) {
       const uint32_t off = (uint32_t)y * pi + x0, noff = (uint32_t)cy * pi + x0;
@@ -266,18 +298,6 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
         march_wall(P, phi, noff, y != cy, sd, u);
 #pragma unroll
         for (int i = 0; i < 19; ++i) pair_value(i, f, gf, gs) = u[i];
-      }
-      uint32_t e[19];
-      float mac5[5];
-      if (odd) {
-        if (pass == 0) {
-          float tf[9], tgf[5], tgs[5];
-          Pops<S, float>::pull(src, pi, pl, nx - 2, nx - 3, nx - 1, cy, cy - 1, cy + 1, inv_scale,
-                               tf, tgf, tgs);
-#pragma unroll
-          for (int i = 0; i < 19; ++i) to[i] = i < 9 ? tf[i] : (i < 14 ? tgf[i - 9] : tgs[i - 14]);
-        }
-        march_odd<S>(P1, phi, off, noff - 1u, scale, tick + (pass > 0), to, e, mac5);
       }
       const Medium<F2> md = phi ? medium_at<F2>(P, ld_f2(phi + off)) : P.um;
       Macro<F2> m;
@@ -298,7 +318,10 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
         for (int i = 0; i < 19; ++i) {
           F2& v = pair_value(i, f, gf, gs);
           PT w = PP::enc(v, scale, kRandom ? rb.next() : 0u);
-          if (odd) w = PP::low(e[i]);
+          if constexpr (kOdd) {
+            const int k = i == 3 ? 0 : i == 6 ? 1 : i == 7 ? 2 : i == 12 ? 3 : 4;
+            if (odd && value_ex(i) < 0) w = PP::low(column.left[k][r - r0]);
+          }
           if (value_ex(i) > 0) w = PP::from_left(w);
           if (value_ex(i) < 0) w = PP::from_right(w);
           if (value_ey(i) >= 0) {
@@ -311,10 +334,12 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
           v = PP::dec(w, inv_scale);
         }
         if (r < r0 + 2) break;  // the line is not full yet
-        if (odd_strip) {
+        if constexpr (kOdd) {
+          if (pr == npairs - 2) {
 #pragma unroll
-          for (int i = 0; i < 19; ++i)
-            to[i] = __shfl_up_sync(0xffffffffu, pair_value(i, f, gf, gs).v.y, 1);
+            for (int i = 0; i < 19; ++i)
+              column.pulled[r - r0 - 2][i] = pair_value(i, f, gf, gs).v.y;
+          }
         }
         if (wall_next) {
 #pragma unroll
@@ -324,15 +349,29 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
         continue;
       }
       if (own && !odd) PairPops<S>::store(dst, pl, off, scale, f, gf, gs, off, tick + 1u);
-      if (own && odd) {
-        for (int i = 0; i < 19; ++i) dst[(uint32_t)i * pl + off] = element<S>(e[i]);
-        if (write_macros)
-          for (int k = 0; k < 5; ++k) mac[(uint32_t)k * pl + off] = mac5[k];
-      }
       if (!wall_next || pass == 2) break;
       y = j == 1 ? 0 : ny - 1;
 #pragma unroll
       for (int i = 0; i < 19; ++i) pair_value(i, f, gf, gs) = t[i];
+    }
+  }
+  if constexpr (kOdd) {
+    const int j0 = r0 + 1, j1 = r1 - 1;  // rows of the second step, wall rows apart
+    if (odd_strip && j0 <= j1) {
+      __syncwarp();
+      const int y = (j0 == 1 ? 0 : j0) + lane;
+      if (y <= (j1 == ny - 2 ? ny - 1 : j1)) {
+        const int cy = min(max(y, 1), ny - 2);
+        const uint32_t off = (uint32_t)y * pi + (nx - 1);
+        float v[19], mac5[5];
+        uint32_t e[19];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) v[i] = column.pulled[cy - j0][i];
+        march_odd<S>(P1, phi, off, (uint32_t)cy * pi + (nx - 2), scale, tick + 1u, v, e, mac5);
+        for (int i = 0; i < 19; ++i) dst[(uint32_t)i * pl + off] = element<S>(e[i]);
+        if (write_macros)
+          for (int k = 0; k < 5; ++k) mac[(uint32_t)k * pl + off] = mac5[k];
+      }
     }
   }
 }
@@ -341,13 +380,13 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
 // row of waves fills up and its last drains in about 0.7 of a segment's
 // time (fitted to sweeps of s: 6, 10, 14, 20 took 84, 88, 91, 106 us a step at
 // 2048^2 FP32, 284, 277, 279, 285 at 4096^2 FP32, and 10, 14, 20, 24 took 1018,
-// 996, 984, 982 at 8192^2 BF16).  Not above 24: the rows in work at one time
+// 996, 984, 982 at 8192^2 BF16).  Not above kMarchRows: the rows in work at one time
 // then spread over more memory than L2 and the address translation hold
 // (4096^2: 404 us with one wave of 98-row segments).
 inline int march_rows(int strips, int ny, int warps) {
   int best = 6;
   double cost = 1e30;
-  for (int s = 6; s <= 24; s += 2) {
+  for (int s = 6; s <= kMarchRows; s += 2) {
     const double waves = (double)strips * ((ny + s - 1) / s) / warps;
     const double c = (waves + 0.7) * (2 * s + 2);
     if (c < cost) {
