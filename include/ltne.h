@@ -245,14 +245,17 @@ int64_t ltne_kernel_launch_count(const ltne_handle* h);
    nodes_per_thread the block shape changes no bit.  Defaults: 32 x 4 with
    two nodes per thread for FP16 / BF16 lattices of 2^20 nodes or more,
    128 x 1 with two for FP32 lattices of 2^22 nodes or more, 64 x 2 with
-   one otherwise (and always for FP64).  With two nodes per thread, cavity
-   walls and no local h_v, lattices of 2^22 nodes or more (FP32) or 2^24
-   (16-bit storage) advance two steps per launch, in strips that do not
-   depend on the block shape; with one (cavity walls, FP32, FP16 or BF16
-   storage), lattices up to about 200 x 200 advance up to four, in tiles, and
-   FP32 lattices of 2^20 nodes or more without local h_v two.  The results are the same bits.  FP64 cavities at the default shape step from a
-   list of nodes in one-warp blocks, again the same bits.  May be called at any
-   time between steps.
+   one otherwise (and always for FP64).  Launches may advance several steps,
+   with the same bits, in kernels that do not depend on the block shape (cavity
+   walls; FP32, FP16 or BF16 storage).  Two nodes per thread, no local h_v: two
+   steps for lattices of 2^22 nodes or more (FP32) or 2^24 (16-bit storage).
+   One node per thread: up to four for lattices up to about 200 x 200, in
+   tiles; two for FP32 lattices of 2^20 nodes or more without local h_v.  A
+   default schedule keeps one step per launch on narrow FP32 lattices (rows
+   below about 256 nodes) that would fill the two-step kernels poorly; a
+   schedule that was set does not.  FP64 cavities at the default shape step
+   from a list of nodes in one-warp blocks, again with the same bits.  May be
+   called at any time between steps.
    LTNE_ERR_INVALID_ARG for other schedules. */
 int ltne_set_schedule(ltne_handle* h, int32_t block_x, int32_t block_y,
                       int32_t nodes_per_thread);

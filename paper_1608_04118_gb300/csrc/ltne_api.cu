@@ -527,6 +527,29 @@ LatticeArgs lattice_args(const ltne_handle* h, int src_buf, int write_macros) {
   return a;
 }
 
+// Whether a two-step walk over n nodes or pairs a row fills its strips well
+// enough to beat the default one-step schedule.  Its last strip may hold a few
+// lanes: where it then takes more strips than the row has warps, narrow FP32
+// lattices lose what the second step gives (64 x 32,032 55 us a step with one
+// step per launch, 68 with the walk; 96 x 21,355 54, 59; pairs: 128 x 32,968 151,
+// 164, 186 x 22,750 133, 140).  One node per thread: from 256 nodes a row on the
+// excess no longer shows (256 x 4161 27.5, 26.9), below it an excess of a sixth
+// is paid for from 2^21 nodes on (213 x 9625 55.4, 51.5, but 213 x 5001 29.9,
+// 32.3).  Pairs: up to a fifth (306 x 13,906 127, 119; 256 x 16,584 119, 123) and
+// lanes up to 7/4 of the pairs (66 x 63,750 207, 225); odd widths, slower in the
+// one-step kernel, always (129 x 32,713 185, 154), as in 16-bit storage, bound by
+// issue in both forms (246 x 68,300 FP16 517, 457).  A schedule that was set
+// decides by itself.
+bool march_fills(const ltne_handle* h) {
+  const ltne_params& p = h->p;
+  if (h->shape_set || p.storage != LTNE_F32) return true;
+  const int n = h->shape.pair ? (p.nx + 1) / 2 : p.nx;
+  const int strips = march_strips(n), warps = (n + 31) / 32;
+  if (h->shape.pair) return p.nx % 2 || (5 * strips <= 6 * warps && 4 * 32 * strips <= 7 * n);
+  return strips <= warps || p.nx >= 256 ||
+         ((int64_t)p.nx * p.ny >= (int64_t)1 << 21 && 6 * strips <= 7 * warps);
+}
+
 // Time steps one launch may advance on this handle (a power of two, so that
 // the launches of a captured graph keep the A-B parity).  Two nodes per
 // thread: two where k_step2_pair (ltne_march.cuh) is the faster form.  Its
@@ -543,10 +566,12 @@ int steps_per_launch(const ltne_handle* h) {
   if (h->slab || h->shape.tma || p.bc != LTNE_BC_CAVITY || p.storage == LTNE_F64) return 1;
   const int64_t nodes = (int64_t)p.nx * p.ny;
   if (h->shape.pair) {
-    return !p.hv_local && nodes >= (int64_t)1 << (p.storage == LTNE_F32 ? 22 : 24) ? 2 : 1;
+    const int64_t from = (int64_t)1 << (p.storage == LTNE_F32 ? 22 : 24);
+    return !p.hv_local && nodes >= from && march_fills(h) ? 2 : 1;
   }
   if (h->shape.tiles.ntx) return kTileSteps;
-  return p.storage == LTNE_F32 && !p.hv_local && nodes >= (int64_t)1 << 20 ? 2 : 1;
+  return p.storage == LTNE_F32 && !p.hv_local && nodes >= (int64_t)1 << 20 && march_fills(h) ? 2
+                                                                                             : 1;
 }
 
 cudaError_t launch_step(ltne_handle* h, int src_buf, int write_macros, cudaStream_t st,
@@ -1291,6 +1316,7 @@ int ltne_set_schedule(ltne_handle* h, int32_t block_x, int32_t block_y,
   h->shape.bx = block_x;
   h->shape.by = block_y;
   h->shape.pair = nodes_per_thread == 2 ? 1 : 0;
+  h->shape_set = 1;
   drop_graphs(h);  // the captured launches carry the old configuration
   return LTNE_OK;
 }

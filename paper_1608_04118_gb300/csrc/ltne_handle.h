@@ -13,6 +13,7 @@ struct ltne_handle {
   cudaStream_t aux_stream = nullptr;  // the adjoint's recompute
   ltne::NodeParams<double> P{};
   ltne::StepShape shape;
+  int shape_set = 0;  // the schedule came from ltne_set_schedule
   // derived lattice values
   double L = 0, nu_f = 0, alpha_f = 0, d_ergun = 0;
   // layout

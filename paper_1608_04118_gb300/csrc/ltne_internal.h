@@ -89,6 +89,13 @@ struct TilePlan {
   int ntx = 0, nty = 0, threads = 0;
 };
 
+// Strips of the two-step walks (ltne_march.cuh) over a row of n nodes or pairs:
+// 32 lanes each, of which the second step takes 30, or 31 at a side.
+constexpr int kMarchLanes = 30;
+inline int march_strips(int n) {
+  return n <= 32 ? 1 : (n - 32 + kMarchLanes - 1) / kMarchLanes + 1;
+}
+
 struct StepShape {
   int bx = 64;
   int by = 2;

@@ -212,7 +212,6 @@ template <> __device__ __forceinline__ float element<float>(uint32_t bits) {
   return __uint_as_float(bits);
 }
 
-constexpr int kMarchPairs = 30;   // pairs of a strip advanced by both steps (of 32 by the first)
 constexpr int kMarchBlocks = 20;  // one-warp blocks per SM (96 registers)
 constexpr int kMarchRows = 24;    // rows of a segment at most (march_rows)
 
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(32, kMarchBlocks) k_step2_pair(
   }
   const int lane = threadIdx.x;
   const int npairs = (nx + 1) >> 1;
-  int pr = blockIdx.x * kMarchPairs + lane;
+  int pr = blockIdx.x * kMarchLanes + lane;
   // the second step needs both neighbouring lanes, except at the lattice's sides
   const bool own = pr < npairs && (lane > 0 || pr == 0) && (lane < 31 || pr == npairs - 1);
   pr = min(pr, npairs - 1);  // lanes beyond the lattice repeat its last pair and store nothing
@@ -402,8 +401,7 @@ cudaError_t launch_step2_pair_t(const LatticeArgs& a, const NodeParams<double>& 
                                 cudaStream_t st) {
   const NodeParams<F2> P = cast_params<F2>(Pd);
   const NodeParams<float> P1 = cast_params<float>(Pd);
-  const int npairs = (a.nx + 1) / 2;
-  const int strips = npairs <= 32 ? 1 : (npairs - 32 + kMarchPairs - 1) / kMarchPairs + 1;
+  const int strips = march_strips((a.nx + 1) / 2);
   const int seg = march_rows(strips, a.ny, kSMs * kMarchBlocks);
   const dim3 grid(strips, (a.ny + seg - 1) / seg);
   if (grid.y > (unsigned)kMaxGridY) return cudaErrorInvalidValue;
@@ -422,7 +420,6 @@ cudaError_t launch_step2_pair_t(const LatticeArgs& a, const NodeParams<double>& 
 // wave of segments.  Measured, us a step, one-step kernel -> this: 1024^2 FP32,
 // per-node porosity, 25.7 -> 24.3, 1448^2 50.2 -> 42.7, 2048 x 2047 96.2 -> 78.2 (724^2
 // 10.9 -> 13.6: too few segments).  The bits of two launches of k_step.
-constexpr int kMarchNodes = 30;
 constexpr int kMarchNodeBlocks = 32;
 constexpr int kMarchNodeRows = 8;
 
@@ -434,7 +431,7 @@ static __global__ void __launch_bounds__(32, kMarchNodeBlocks) k_step2_node(
   __shared__ float line[19][32];  // the slots of k_step2_pair
   grid_dep_wait();
   const int lane = threadIdx.x;
-  int x = blockIdx.x * kMarchNodes + lane;
+  int x = blockIdx.x * kMarchLanes + lane;
   const bool own = x < nx && (lane > 0 || x == 0) && (lane < 31 || x == nx - 1);
   x = min(x, nx - 1);
   const int side = x == 0 ? 0 : (x == nx - 1 ? 1 : -1);
@@ -502,7 +499,7 @@ static __global__ void __launch_bounds__(32, kMarchNodeBlocks) k_step2_node(
 
 inline cudaError_t launch_step2_node(const LatticeArgs& a, const NodeParams<double>& Pd,
                                      cudaStream_t st) {
-  const int strips = a.nx <= 32 ? 1 : (a.nx - 32 + kMarchNodes - 1) / kMarchNodes + 1;
+  const int strips = march_strips(a.nx);
   const dim3 grid(strips, (a.ny + kMarchNodeRows - 1) / kMarchNodeRows);
   if (grid.y > (unsigned)kMaxGridY) return cudaErrorInvalidValue;
   return launch_kernel(a.chained != 0, k_step2_node, grid, dim3(32), 0, st,
