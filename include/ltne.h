@@ -418,10 +418,11 @@ size_t ltne_adjoint_workspace_bytes(const ltne_handle* h, int64_t n_steps, int32
    counterpart in the paper).  LTNE_ADJ_ONE_WAVE: every register the kernel
    wants (128 per thread in FP32), for lattices whose grid fits one wave of
    the device, where a reverse step's time is one thread's latency;
-   LTNE_ADJ_CAPPED: registers capped at 80 so that 768 threads share an SM
-   (FP32; a few values spill to local memory), for larger
-   lattices, where occupancy hides the latency.  LTNE_ADJ_AUTO (default)
-   picks by the lattice size.  The two builds run the same code; they agree
+   LTNE_ADJ_CAPPED: registers capped at 80 so that 768 threads share an SM,
+   at 72 and 896 from 2^20 nodes on (FP32; a few values spill to local
+   memory), for larger lattices, where occupancy hides the latency.
+   LTNE_ADJ_AUTO (default) picks by the lattice size.  The builds run the same
+   code; they agree
    to rounding (under the cap the compiler may contract a different set of
    multiply-adds), and each is deterministic.  LTNE_ERR_INVALID_ARG for
    other values. */

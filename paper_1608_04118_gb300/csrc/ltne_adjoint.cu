@@ -260,12 +260,15 @@ __global__ void __launch_bounds__(256) k_adj_seed(const C* __restrict__ SN, C* _
 
 // R2: transposed streaming (gather from y + e_i) and transposed collision;
 // a wall node's thread then folds its result (R1) unless S_n is the initial
-// state (fold = 0), whose wall nodes were not rebuilt.  Two builds of the same
-// code: kCapped = false for lattices that fit one wave, where the kernel's
-// time is one thread's latency; kCapped = true with registers capped at 80,
-// 768 threads per SM (FP32), for larger lattices, where occupancy hides it
-// (at 72 and 64 registers the spills cost more: 400^2 x 100 steps 2.82 and 2.70
-// against 2.56 ms).
+// state (fold = 0), whose wall nodes were not rebuilt.  Three builds of the same
+// code, by the blocks of 128 threads that the registers leave an SM (FP32): 4
+// for lattices that fit one wave, where the kernel's time is one thread's
+// latency; for larger ones, where occupancy hides it, 6 (at most 80 registers),
+// and from 2^20 nodes on, bound by HBM, 7 (72).  Whole calls with 6, 7 and 8 blocks:
+// 400^2 x 100 steps 2.52, 2.59, 2.63 ms, 724^2 x 100 6.29, 6.35, 6.56, 1024^2 x 60
+// 7.33, 7.28, 7.34, 2048^2 x 60 27.04, 26.78, 26.86.  The capped builds load the
+// recorded state after the folds, which leaves them the registers: before them,
+// 6 and 7 blocks took 2.56 and 2.85 at 400^2, 27.11 and 28.96 at 2048^2.
 //
 // The one-wave build loads the recorded state, also a wall node's source,
 // before it waits for the previous reverse step, and lets the next step's
@@ -278,8 +281,10 @@ __global__ void __launch_bounds__(256) k_adj_seed(const C* __restrict__ SN, C* _
 // the wait as well gave 4.36 at 256^2, but other contractions (dJ/dphi 2e-6
 // apart); on larger lattices what is held across the wait costs occupancy
 // (1024^2 12.0 -> 13.4 ms), so the capped build waits first.
-template <typename C, bool kCapped>
-__global__ void __launch_bounds__(128, sizeof(C) == 8 ? 1 : kCapped ? 6 : 4)
+constexpr int kAdjOneWave = 4, kAdjCapped = 6, kAdjCappedLarge = 7;  // blocks per SM
+
+template <typename C, int kBlocks>
+__global__ void __launch_bounds__(128, sizeof(C) == 8 ? 1 : kBlocks)
     k_adj_main(const C* __restrict__ Lam,
                                                   C* __restrict__ lam_out,
                                                   const C* __restrict__ S,
@@ -288,6 +293,7 @@ __global__ void __launch_bounds__(128, sizeof(C) == 8 ? 1 : kCapped ? 6 : 4)
                                                   C* __restrict__ wphib, const NodeParams<C> P,
                                                   int nx, int ny, int64_t pitch, int64_t plane,
                                                   int fold, const C* __restrict__ S_prev) {
+  constexpr bool kCapped = kBlocks != kAdjOneWave;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= nx || y >= ny) {
@@ -335,13 +341,13 @@ __global__ void __launch_bounds__(128, sizeof(C) == 8 ? 1 : kCapped ? 6 : 4)
       qgs[i] = pulled ? Lam[(int64_t)(14 + i) * plane + toff] : C(0);
     }
   }
+  if (x <= 2 || x >= nx - 3 || y <= 2 || y >= ny - 3)
+    add_wall_folds<!kCapped && sizeof(C) == 4>(Lam, x, y, nx, ny, pitch, plane, qf, qgf, qgs);
   if (kCapped) {
+    if (wall) load_wall_source(S, phi, x, y, nx, ny, pitch, plane, w);
     load19(S, plane, off, f, gf, gs);
     ph = phi[off];
   }
-  if (x <= 2 || x >= nx - 3 || y <= 2 || y >= ny - 3)
-    add_wall_folds<!kCapped && sizeof(C) == 4>(Lam, x, y, nx, ny, pitch, plane, qf, qgf, qgs);
-  if (kCapped && wall) load_wall_source(S, phi, x, y, nx, ny, pitch, plane, w);
   const Medium<C> md = medium_at<C>(P, ph);
   C fb[9] = {}, gfb[5] = {}, gsb[5] = {};
   MediumBar<C> mdb;
@@ -646,11 +652,16 @@ int run_adjoint(ltne_handle* h, const double* porosity, const double* rho, const
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_main<C, false>,
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_main<C, kAdjOneWave>,
                                                         (int)(blk.x * blk.y), 0);
     if (e != cudaSuccess) return LTNE_ERR_CUDA;
     capped = (int64_t)grd.x * grd.y > (int64_t)sms * per_sm;
   }
+  // (FP64 has one capped build: its registers are never capped)
+  constexpr int kLarge = sizeof(C) == 4 ? kAdjCappedLarge : kAdjCapped;
+  const auto adj_main = !capped                                ? k_adj_main<C, kAdjOneWave>
+                        : (int64_t)nx * ny >= (int64_t)1 << 20 ? k_adj_main<C, kLarge>
+                                                               : k_adj_main<C, kAdjCapped>;
   // Slot set q holds a segment's states: slot 0 (S_a, copied from its
   // checkpoint) and K recomputed slots.  The sweep reverses segment s from
   // one set while segment s - 1 is recomputed into the other on a second
@@ -692,14 +703,8 @@ int run_adjoint(ltne_handle* h, const double* porosity, const double* rho, const
     for (int64_t j = len - 1; j >= 0 && le == cudaSuccess; --j) {
       const int fold = (initial && j == 0) ? 0 : 1;
       const C* pre = j > 0 ? slot(q, j - 1) : nullptr;
-      if (capped)
-        le = launch_chained(chained, k_adj_main<C, true>, grd, blk, s_, (const C*)lL, lO,
-                            (const C*)slot(q, j), phi, phib, hb, wphib, P, nx, ny, pitch, plane,
-                            fold, pre);
-      else
-        le = launch_chained(chained, k_adj_main<C, false>, grd, blk, s_, (const C*)lL, lO,
-                            (const C*)slot(q, j), phi, phib, hb, wphib, P, nx, ny, pitch, plane,
-                            fold, pre);
+      le = launch_chained(chained, adj_main, grd, blk, s_, (const C*)lL, lO, (const C*)slot(q, j),
+                          phi, phib, hb, wphib, P, nx, ny, pitch, plane, fold, pre);
       chained = true;
       C* t = lL;
       lL = lO;

@@ -536,7 +536,7 @@ class Cavity:
 
     def set_adjoint_schedule(self, mode):
         """Register budget of the adjoint's transposed collision: 0 by lattice
-        size, 1 all registers (one wave), 2 capped (80 registers)."""
+        size, 1 all registers (one wave), 2 capped (80 registers, 72 from 2^20 nodes)."""
         ltne_set_adjoint_schedule(self.h, mode)
         return self
 
