@@ -153,12 +153,16 @@ template <> LTNE_HD double csqrt_<double>(double x) { return sqrt(x); }
 
 // |u| over FP32's whole range, given the value mag that sqrt_ makes of its
 // square, which is 0 where the square is below the normal range: what Eq. 52
-// takes, whose power 0.644 makes 1e-13 of a speed of 1e-20.
+// takes, whose power 0.644 makes 1e-13 of a speed of 1e-20.  The step kernels
+// have instantiations of their own for the local h_v (kHv), which differ from
+// the others in this alone: beside the plain step it cost registers (2049 x 1531
+// BF16 60.4 -> 61.8 us a step), and under the branch on P.hv_local its latency
+// (600 x 400 FP16 with the local h_v 7.97 -> 8.18; without the branch 7.97).
 template <typename C> LTNE_HD C full_speed(C mag, C, C) { return mag; }
 template <> LTNE_HD float full_speed<float>(float mag, float ux, float uy) {
-  if (mag != 0.0f || (ux == 0.0f && uy == 0.0f)) return mag;
-  const float x = 0x1p100f * ux, y = 0x1p100f * uy;  // both below 2^-62 before
-  return 0x1p-100f * sqrt_<float>(x * x + y * y);
+  const float x = 0x1p100f * ux, y = 0x1p100f * uy;  // taken for |ux|, |uy| < 2^-62
+  const float t = 0x1p-100f * sqrt_<float>(x * x + y * y);
+  return mag == 0.0f ? t : mag;
 }
 
 // The coefficients at porosity phi (per-node porosity fields).

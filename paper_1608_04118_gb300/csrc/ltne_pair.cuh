@@ -232,7 +232,7 @@ __device__ __forceinline__ void st_f2(float* __restrict__ p, F2 v) {
 // Everything after the pull for a pair at element offset off whose
 // pre-collision values are in f, gf, gs: macroscopic values, collision,
 // stores.  Shared by the pull from HBM and the pull from a staged tile.
-template <typename S>
+template <typename S, bool kHv = false>
 __device__ __forceinline__ void finish_pair(S* __restrict__ dst,
                                             const float* __restrict__ phi_field,
                                             float* __restrict__ mac, const NodeParams<F2>& P,
@@ -245,7 +245,7 @@ __device__ __forceinline__ void finish_pair(S* __restrict__ dst,
   if (P.hv_local) set_exchange<F2>(md, hv_local_at<F2>(P, ld_f2(um_in + off)));
   Macro<F2> m;
   macros<F2>(P, md, f, gf, gs, m);
-  if (P.hv_local) st_f2(um_out + off, full_speed<F2>(m.umag, m.ux, m.uy));
+  if (kHv || P.hv_local) st_f2(um_out + off, kHv ? full_speed<F2>(m.umag, m.ux, m.uy) : m.umag);
   if (write_macros) {
     st_f2(mac + off, m.drho);
     st_f2(mac + pl + off, m.ux);
@@ -260,7 +260,7 @@ __device__ __forceinline__ void finish_pair(S* __restrict__ dst,
 // The pair (x0, y), (x0 + 1, y) when both nodes exist and neither is a
 // left/right wall node: interior nodes, or both on a no-slip adiabatic row
 // (same rebuild, from the row above or below).
-template <typename S, int BC>
+template <typename S, int BC, bool kHv = false>
 __device__ __forceinline__ void step_pair(const S* __restrict__ src, S* __restrict__ dst,
                                           const float* __restrict__ phi_field,
                                           float* __restrict__ mac, const NodeParams<F2>& P,
@@ -298,8 +298,8 @@ __device__ __forceinline__ void step_pair(const S* __restrict__ src, S* __restri
     macros<F2>(P, mdn, f, gf, gs, mn);
     nee<F2>(P, mn, mn.dTf, mn.dTs, f, gf, gs);  // adiabatic: the neighbour's temperatures
   }
-  finish_pair<S>(dst, phi_field, mac, P, off, pl, scale, write_macros, tick, um_in, um_out, f, gf,
-                 gs);
+  finish_pair<S, kHv>(dst, phi_field, mac, P, off, pl, scale, write_macros, tick, um_in, um_out, f,
+                      gf, gs);
 }
 
 // A cavity pair holding a left or right wall node (x0 = 0, or x0 + 1 =
@@ -312,7 +312,7 @@ __device__ __forceinline__ void step_pair(const S* __restrict__ src, S* __restri
 // lanes continue as any pair.  The same rebuild as the one-node step, in
 // paired arithmetic, without the warp divergence of two one-node steps
 // beside the pairs of the rest of the row.
-template <typename S>
+template <typename S, bool kHv = false>
 __device__ __forceinline__ void step_pair_side(const S* __restrict__ src, S* __restrict__ dst,
                                                const float* __restrict__ phi_field,
                                                float* __restrict__ mac, const NodeParams<F2>& P,
@@ -379,8 +379,8 @@ __device__ __forceinline__ void step_pair_side(const S* __restrict__ src, S* __r
     gs[i] = pick(rgs[i], gs[i]);
   }
   const uint32_t off = (uint32_t)y * pi + (uint32_t)x0;
-  finish_pair<S>(dst, phi_field, mac, P, off, pl, scale, write_macros, tick, um_in, um_out, f, gf,
-                 gs);
+  finish_pair<S, kHv>(dst, phi_field, mac, P, off, pl, scale, write_macros, tick, um_in, um_out, f,
+                      gf, gs);
 }
 
 // Register budget of the pair kernel: blocks of at most 128 threads and at
@@ -392,7 +392,7 @@ __device__ __forceinline__ void step_pair_side(const S* __restrict__ src, S* __r
 constexpr int kPairMaxThreads = kPairBlockThreads;
 constexpr int kPairMinBlocks = 5;
 
-template <typename S, int BC>
+template <typename S, int BC, bool kHv>
 __global__ void __launch_bounds__(kPairMaxThreads, kPairMinBlocks) k_step_pair(
     const S* __restrict__ src, S* __restrict__ dst, const float* __restrict__ phi_field,
     float* __restrict__ mac, const NodeParams<F2> P, const NodeParams<float> P1, const int nx,
@@ -407,17 +407,17 @@ __global__ void __launch_bounds__(kPairMaxThreads, kPairMinBlocks) k_step_pair(
   const bool full = x0 + 1 < nx;
   const bool uniform = BC == BC_CAVITY ? (x0 > 0 && x0 + 2 < nx) : full;
   if (uniform) {
-    step_pair<S, BC>(src, dst, phi_field, mac, P, x0, y, nx, ny, (uint32_t)pitch,
-                     (uint32_t)plane, scale, inv_scale, write_macros, tick, um_in, um_out);
+    step_pair<S, BC, kHv>(src, dst, phi_field, mac, P, x0, y, nx, ny, (uint32_t)pitch,
+                          (uint32_t)plane, scale, inv_scale, write_macros, tick, um_in, um_out);
   } else if (BC == BC_CAVITY && full) {
-    step_pair_side<S>(src, dst, phi_field, mac, P, x0, y, nx, ny, (uint32_t)pitch,
-                      (uint32_t)plane, scale, inv_scale, write_macros, tick, um_in, um_out);
+    step_pair_side<S, kHv>(src, dst, phi_field, mac, P, x0, y, nx, ny, (uint32_t)pitch,
+                           (uint32_t)plane, scale, inv_scale, write_macros, tick, um_in, um_out);
   } else {
-    step_node<S, float, BC>(src, dst, phi_field, mac, P1, x0, y, nx, ny, pitch, plane, scale,
-                            inv_scale, write_macros, tick, nullptr, um_in, um_out);
+    step_node<S, float, BC, kHv>(src, dst, phi_field, mac, P1, x0, y, nx, ny, pitch, plane, scale,
+                                 inv_scale, write_macros, tick, nullptr, um_in, um_out);
     if (full)
-      step_node<S, float, BC>(src, dst, phi_field, mac, P1, x0 + 1, y, nx, ny, pitch, plane,
-                              scale, inv_scale, write_macros, tick, nullptr, um_in, um_out);
+      step_node<S, float, BC, kHv>(src, dst, phi_field, mac, P1, x0 + 1, y, nx, ny, pitch, plane,
+                                   scale, inv_scale, write_macros, tick, nullptr, um_in, um_out);
   }
 }
 
@@ -437,11 +437,13 @@ cudaError_t launch_step_pair_t(const LatticeArgs& a, const NodeParams<double>& P
   float* mac = static_cast<float*>(a.mac);
   const float* um_in = static_cast<const float*>(a.um_in);
   float* um_out = static_cast<float*>(a.um_out);
+  const bool hv = Pd.hv_local != 0;
   cudaError_t e;
 #define LTNE_PAIR_LAUNCH(bc)                                                                   \
-  e = launch_kernel(a.chained != 0, k_step_pair<S, bc>, grid, block, 0, st, src, dst, phi,     \
-                    mac, P, P1, a.nx, a.ny, a.pitch, a.plane, scale, inv_scale,                \
-                    a.write_macros, a.tick_in, a.tick_out, um_in, um_out)
+  e = launch_kernel(a.chained != 0, hv ? k_step_pair<S, bc, true> : k_step_pair<S, bc, false>, \
+                    grid, block, 0, st, src, dst, phi, mac, P, P1, a.nx, a.ny, a.pitch,        \
+                    a.plane, scale, inv_scale, a.write_macros, a.tick_in, a.tick_out, um_in,   \
+                    um_out)
   switch (a.bc) {
     case BC_CAVITY: LTNE_PAIR_LAUNCH(BC_CAVITY); break;
     case BC_PERIODIC: LTNE_PAIR_LAUNCH(BC_PERIODIC); break;

@@ -176,7 +176,7 @@ __device__ __forceinline__ void update_node(const NodeParams<C>& P,
 
 // One node (x, y) of one time step: pull, wall rebuild, macroscopic values,
 // collision, store.  Shared by the single-lattice and the batched kernels.
-template <typename S, typename C, int BC>
+template <typename S, typename C, int BC, bool kHv = false>
 __device__ __forceinline__ void step_node(const S* __restrict__ src, S* __restrict__ dst,
                                           const C* __restrict__ phi_field, C* __restrict__ mac,
                                           const NodeParams<C>& P, const int x, const int y,
@@ -227,7 +227,7 @@ __device__ __forceinline__ void step_node(const S* __restrict__ src, S* __restri
   update_node<C, BC>(P, phi_field, off, noff, kind, um_in + off, um_in + noff, plane, pre_out, f,
                      gf, gs, m);
   // u_m of Eq. 52 for the next state
-  if (P.hv_local) um_out[off] = full_speed<C>(m.umag, m.ux, m.uy);
+  if (kHv || P.hv_local) um_out[off] = kHv ? full_speed<C>(m.umag, m.ux, m.uy) : m.umag;
   if (write_macros) store_macros<C>(mac, plane, off, m);
   Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, (uint32_t)off, tick);
 }
@@ -247,7 +247,7 @@ __device__ __forceinline__ uint32_t read_tick(const uint32_t* __restrict__ tick_
   return tick;
 }
 
-template <typename S, typename C, int BC>
+template <typename S, typename C, int BC, bool kHv>
 __global__ void __launch_bounds__(256) k_step(const S* __restrict__ src, S* __restrict__ dst,
                                               const C* __restrict__ phi_field,
                                               C* __restrict__ mac, const NodeParams<C> P,
@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(256) k_step(const S* __restrict__ src, S* __re
   if (BC == BC_SLAB && ((y == 0 && !(slab_walls & SLAB_LO_WALL)) ||
                         (y == ny - 1 && !(slab_walls & SLAB_HI_WALL))))
     return;  // a halo row: the neighbouring slab's values, read only
-  step_node<S, C, BC>(src, dst, phi_field, mac, P, x, y, nx, ny, pitch, plane, scale, inv_scale,
-                      write_macros, tick, nullptr, um_in, um_out, slab_walls);
+  step_node<S, C, BC, kHv>(src, dst, phi_field, mac, P, x, y, nx, ny, pitch, plane, scale,
+                           inv_scale, write_macros, tick, nullptr, um_in, um_out, slab_walls);
 }
 
 // One step of a cavity from a list of its nodes in blocks of one warp: the
@@ -374,10 +374,14 @@ cudaError_t launch_step_t(const LatticeArgs& a, const NodeParams<double>& Pd, St
                            inv_scale, a.write_macros, um_in, um_out);
     }
   }
+  // (FP64 needs no kHv kernels, and slabs take no local h_v)
+  constexpr bool kHv = sizeof(C) == 4;
+  const bool hv = Pd.hv_local != 0;
 #define LTNE_STEP_LAUNCH(bc, walls)                                                            \
-  e = launch_kernel(ch, k_step<S, C, bc>, g, b, 0, st, src, dst, phi, mac, P, a.nx, a.ny,       \
-                    a.pitch, a.plane, scale, inv_scale, a.write_macros, a.tick_in, a.tick_out,  \
-                    um_in, um_out, walls)
+  e = launch_kernel(ch, hv && bc != BC_SLAB ? k_step<S, C, bc, kHv && bc != BC_SLAB>           \
+                                            : k_step<S, C, bc, false>,                         \
+                    g, b, 0, st, src, dst, phi, mac, P, a.nx, a.ny, a.pitch, a.plane, scale,   \
+                    inv_scale, a.write_macros, a.tick_in, a.tick_out, um_in, um_out, walls)
   switch (a.bc) {
     case BC_CAVITY: LTNE_STEP_LAUNCH(BC_CAVITY, 0); break;
     case BC_PERIODIC: LTNE_STEP_LAUNCH(BC_PERIODIC, 0); break;

@@ -38,7 +38,7 @@ struct TileSmem {
   C um[2][kTileNodes];        // |u| (local h_v)
 };
 
-template <typename S, typename C>
+template <typename S, typename C, bool kHv>
 __global__ void __launch_bounds__(kTileThreads) k_step_tile(
     const S* __restrict__ src, S* __restrict__ dst, const C* __restrict__ phi, C* __restrict__ mac,
     const __grid_constant__ NodeParams<C> P, const int nx, const int ny, const int64_t pitch,
@@ -93,11 +93,11 @@ __global__ void __launch_bounds__(kTileThreads) k_step_tile(
       Macro<C> m;
       update_node<C, BC_CAVITY>(P, phi, off, noff, kind, um, umn, 0, nullptr, f, gf, gs, m);
       if (e == 0) {
-        if (P.hv_local) um_out[off] = full_speed<C>(m.umag, m.ux, m.uy);
+        if (kHv || P.hv_local) um_out[off] = kHv ? full_speed<C>(m.umag, m.ux, m.uy) : m.umag;
         if (write_macros) store_macros<C>(mac, plane, off, m);
         Pops<S, C>::store(dst, plane, off, scale, f, gf, gs, off, tick + s);
       } else {
-        if (P.hv_local) sm.um[out][q] = full_speed<C>(m.umag, m.ux, m.uy);
+        if (kHv || P.hv_local) sm.um[out][q] = kHv ? full_speed<C>(m.umag, m.ux, m.uy) : m.umag;
         Pops<S, C>::store(&sm.pops[out][0][0], kTileNodes, q, scale, f, gf, gs, off, tick + s);
       }
     }
@@ -130,7 +130,7 @@ cudaError_t launch_step_tile_t(const LatticeArgs& a, const NodeParams<double>& P
                                const StepShape& shape, cudaStream_t st) {
   const TilePlan& p = shape.tiles;
   if (shape.steps > kTileSteps || !p.ntx || a.bc != BC_CAVITY) return cudaErrorInvalidValue;
-  const auto k = k_step_tile<S, C>;
+  const auto k = Pd.hv_local ? k_step_tile<S, C, true> : k_step_tile<S, C, false>;
   constexpr int bytes = (int)sizeof(TileSmem<S, C>);
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;

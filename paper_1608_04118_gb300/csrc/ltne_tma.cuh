@@ -136,7 +136,7 @@ __device__ __forceinline__ void pull_staged(const S* __restrict__ sb, int r, int
   }
 }
 
-template <typename S, int TX, int TY, int NS>
+template <typename S, int TX, int TY, int NS, bool kHv>
 __global__ void __launch_bounds__(TX * TY, kPairMinBlocks) k_step_tma(
     const __grid_constant__ CUtensorMap tmap, const S* __restrict__ src, S* __restrict__ dst,
     const float* __restrict__ phi_field, float* __restrict__ mac, const NodeParams<F2> P,
@@ -199,17 +199,18 @@ __global__ void __launch_bounds__(TX * TY, kPairMinBlocks) k_step_tma(
       F2 f[9], gf[5], gs[5];
       pull_staged<S, B::BW, B::kPlane>(sb, (int)threadIdx.y + 1, B::A + 2 * (int)threadIdx.x,
                                        inv_scale, f, gf, gs);
-      finish_pair<S>(dst, phi_field, mac, P, (uint32_t)y * pi + (uint32_t)x0, pl, scale,
-                     write_macros, tick, um_in, um_out, f, gf, gs);
+      finish_pair<S, kHv>(dst, phi_field, mac, P, (uint32_t)y * pi + (uint32_t)x0, pl, scale,
+                          write_macros, tick, um_in, um_out, f, gf, gs);
     } else if (x0 > 0 && x0 + 2 < nx) {  // both nodes on a wall row
-      step_pair<S, BC_CAVITY>(src, dst, phi_field, mac, P, x0, y, nx, ny, pi, pl, scale,
-                              inv_scale, write_macros, tick, um_in, um_out);
+      step_pair<S, BC_CAVITY, kHv>(src, dst, phi_field, mac, P, x0, y, nx, ny, pi, pl, scale,
+                                   inv_scale, write_macros, tick, um_in, um_out);
     } else if (x0 + 1 < nx) {  // a wall column in the pair
-      step_pair_side<S>(src, dst, phi_field, mac, P, x0, y, nx, ny, pi, pl, scale, inv_scale,
-                        write_macros, tick, um_in, um_out);
+      step_pair_side<S, kHv>(src, dst, phi_field, mac, P, x0, y, nx, ny, pi, pl, scale, inv_scale,
+                             write_macros, tick, um_in, um_out);
     } else {  // the last node of an odd row
-      step_node<S, float, BC_CAVITY>(src, dst, phi_field, mac, P1, x0, y, nx, ny, pitch, plane,
-                                     scale, inv_scale, write_macros, tick, nullptr, um_in, um_out);
+      step_node<S, float, BC_CAVITY, kHv>(src, dst, phi_field, mac, P1, x0, y, nx, ny, pitch, plane,
+                                          scale, inv_scale, write_macros, tick, nullptr, um_in,
+                                          um_out);
     }
   }
 }
@@ -271,7 +272,7 @@ cudaError_t make_tile_map(CUtensorMap* map, const void* base, int64_t pitch, int
 #define LTNE_TMA_STAGES 2
 #endif
 
-template <typename S, int TX, int TY>
+template <typename S, int TX, int TY, bool kHv>
 cudaError_t launch_tma_shape(const LatticeArgs& a, const NodeParams<double>& Pd,
                              cudaStream_t st) {
   constexpr int NS = LTNE_TMA_STAGES;
@@ -289,11 +290,11 @@ cudaError_t launch_tma_shape(const LatticeArgs& a, const NodeParams<double>& Pd,
     TmaLaunchInfo& li = info[dev];
     if (!li.blocks_per_sm) {
       int nb = 0, n_sm = 0;
-      if (cudaFuncSetAttribute(k_step_tma<S, TX, TY, NS>,
+      if (cudaFuncSetAttribute(k_step_tma<S, TX, TY, NS, kHv>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                B::kSmem) != cudaSuccess ||
           cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_tma<S, TX, TY, NS>, TX * TY,
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_tma<S, TX, TY, NS, kHv>, TX * TY,
                                                         B::kSmem) != cudaSuccess ||
           nb < 1)
         return cudaErrorInvalidConfiguration;
@@ -307,7 +308,7 @@ cudaError_t launch_tma_shape(const LatticeArgs& a, const NodeParams<double>& Pd,
   const int grid = ntiles < blocks_per_sm * sms ? ntiles : blocks_per_sm * sms;
   const NodeParams<F2> P = cast_params<F2>(Pd);
   const NodeParams<float> P1 = cast_params<float>(Pd);
-  k_step_tma<S, TX, TY, NS><<<grid, dim3(TX, TY), B::kSmem, st>>>(
+  k_step_tma<S, TX, TY, NS, kHv><<<grid, dim3(TX, TY), B::kSmem, st>>>(
       map, static_cast<const S*>(a.src), static_cast<S*>(a.dst),
       static_cast<const float*>(a.phi), static_cast<float*>(a.mac), P, P1, a.nx, a.ny, a.pitch,
       a.plane, a.enc_scale, 1.0f / a.enc_scale, a.write_macros, a.tick_in, a.tick_out,
@@ -317,13 +318,19 @@ cudaError_t launch_tma_shape(const LatticeArgs& a, const NodeParams<double>& Pd,
 
 // The staged kernel's tile follows the schedule's block shape: 32 x 4,
 // 64 x 2 or 32 x 2 threads (any other shape runs as 32 x 4).
+template <typename S, bool kHv>
+cudaError_t launch_tma(const LatticeArgs& a, const NodeParams<double>& Pd, StepShape s,
+                       cudaStream_t st) {
+  if (s.bx == 64 && s.by == 2) return launch_tma_shape<S, 64, 2, kHv>(a, Pd, st);
+  if (s.bx == 32 && s.by == 2) return launch_tma_shape<S, 32, 2, kHv>(a, Pd, st);
+  return launch_tma_shape<S, 32, 4, kHv>(a, Pd, st);
+}
+
 template <typename S>
 cudaError_t launch_step_tma_t(const LatticeArgs& a, const NodeParams<double>& Pd, StepShape s,
                               cudaStream_t st) {
   if (a.bc != BC_CAVITY || !a.err) return cudaErrorInvalidValue;
-  if (s.bx == 64 && s.by == 2) return launch_tma_shape<S, 64, 2>(a, Pd, st);
-  if (s.bx == 32 && s.by == 2) return launch_tma_shape<S, 32, 2>(a, Pd, st);
-  return launch_tma_shape<S, 32, 4>(a, Pd, st);
+  return Pd.hv_local ? launch_tma<S, true>(a, Pd, s, st) : launch_tma<S, false>(a, Pd, s, st);
 }
 
 }  // namespace ltne
