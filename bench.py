@@ -174,8 +174,10 @@ def step_kernel(storage, schedule, staged, n, steps, launches):
     """The kernel that made the timed steps of an n x n cavity with per-node
     porosity: by the schedule (block_x, block_y, nodes per thread), whether
     tiles were staged, and whether its launches advanced more than a step."""
-    if launches < steps:  # one node per thread: tiles up to about 200 x 200, the walk from 1024 x 1024
-        return "k_step2_pair" if schedule[2] == 2 else "k_step2_node" if n >= 1024 else "k_step_tile"
+    if launches < steps:
+        if schedule[2] == 2:
+            return "k_step2_pair"
+        return "k_step2_node" if n >= 1024 else "k_step_tile"  # tiles: up to about 200 x 200
     if staged:
         return "k_step_tma"
     if storage == "f64" and tuple(schedule[:2]) == (64, 2):

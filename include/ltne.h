@@ -230,7 +230,8 @@ int ltne_get_state(ltne_handle* h, void* host, size_t bytes);
 int ltne_set_state(ltne_handle* h, const void* host, size_t bytes);
 
 /* Number of time steps issued as step-kernel launches by this handle so far:
-   one per step, also where one launch advances two (see ltne_set_schedule).
+   one per step, also where one launch advances several (see
+   ltne_set_schedule).
    ltne_kernel_launch_count: the launches themselves. */
 int64_t ltne_launch_count(const ltne_handle* h);
 int64_t ltne_kernel_launch_count(const ltne_handle* h);

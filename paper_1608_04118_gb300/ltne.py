@@ -486,7 +486,7 @@ class Cavity:
 
     @property
     def kernel_launches(self):
-        """Step-kernel launches (a launch may advance two steps)."""
+        """Step-kernel launches (a launch may advance several steps)."""
         return ltne_kernel_launch_count(self.h)
 
     def set_schedule(self, block_x, block_y, nodes_per_thread):
