@@ -557,9 +557,9 @@ bool march_fills(const ltne_handle* h) {
 // 2^22 nodes (2048^2 96 -> 84 us a step; 1024^2 27 -> 30), 16-bit storage from
 // 2^24 (4096^2 FP16 307 -> 296; 2048^2 82 -> 92).  One node per thread, FP32
 // arithmetic: four where one block per SM holds the lattice in tiles of
-// k_step_tile (ltne_tile.cuh; up to about 200 x 200: 192^2 2.37 -> 2.18; with
+// k_step_tile (ltne_tile.cuh; up to about 200 x 200: 192^2 2.44 -> 2.24; with
 // two blocks per SM 256^2 2.88 -> 2.95); two by k_step2_node for FP32 from 2^20
-// (1024^2 25.7 -> 24.3, 1448^2 50 -> 43; 724^2 10.9 -> 13.6; the 16-bit forms are
+// (1024^2 25.7 -> 24.7, 1448^2 50 -> 43; 724^2 10.9 -> 13.6; the 16-bit forms are
 // bound by issue already).
 int steps_per_launch(const ltne_handle* h) {
   const ltne_params& p = h->p;

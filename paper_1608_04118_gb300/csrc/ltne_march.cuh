@@ -17,14 +17,14 @@
 // What it pays: the first step of a strip's two outer pairs and of the rows
 // below and above a segment is made twice, once by each neighbour (about
 // (seg + 2) / seg * 32 / 30 of the first steps).  Bound: 16-bit storage, the
-// FMA pipe (busy 69 % of the cycles at 4096^2: a paired instruction holds it
-// for two), with 63 % of the issue slots taken; FP32, that and the rows' loads
-// (DRAM at 70 % of the copy).  Measured, us a step, one-step kernel -> this:
-//   4096^2 FP32, per-node porosity   374 -> 278  (60.2 GLUPS)
+// FMA pipe (busy 70 % of the cycles at 4096^2: a paired instruction holds it
+// for two), with 64 % of the issue slots taken; FP32, that (57 and 52 %) and the
+// rows' loads (DRAM at 76 % of the copy).  Measured, us a step, one-step kernel -> this:
+//   4096^2 FP32, per-node porosity   374 -> 279  (60.2 GLUPS)
 //   2048^2 FP32, per-node porosity    96 -> 84
-//   8192^2 FP16, uniform porosity   1003 -> 964  (69.6 GLUPS)
-//   8192^2 FP16, per-node porosity  1205 -> 1068
-//   8192^2 BF16, per-node porosity  1132 -> 987
+//   8192^2 FP16, uniform porosity   1000 -> 963  (69.7 GLUPS)
+//   8192^2 FP16, per-node porosity  1206 -> 1075
+//   8192^2 BF16, per-node porosity  1135 -> 996
 // One warp per block: blocks of four warps keep the slots of finished warps
 // (4096^2: 287).  20 blocks per SM, 96 registers: at 80 registers and 24
 // blocks the spills cost more than the warps give (348).  The next row's
@@ -418,7 +418,7 @@ cudaError_t launch_step2_pair_t(const LatticeArgs& a, const NodeParams<double>& 
 // 24.6, 28.1 us a step at 1024^2, 82, 79, 78, 79, 79 at 2048 x 2047).  64 registers,
 // 32 one-warp blocks per SM.  Bound: instruction issue, and at 1024^2 the last
 // wave of segments.  Measured, us a step, one-step kernel -> this: 1024^2 FP32,
-// per-node porosity, 25.7 -> 24.3, 1448^2 50.2 -> 42.7, 2048 x 2047 96.2 -> 78.2 (724^2
+// per-node porosity, 25.7 -> 24.7, 1448^2 50.3 -> 43.1, 2048 x 2047 96.0 -> 78.5 (724^2
 // 10.9 -> 13.6: too few segments).  The bits of two launches of k_step.
 constexpr int kMarchNodeBlocks = 32;
 constexpr int kMarchNodeRows = 8;

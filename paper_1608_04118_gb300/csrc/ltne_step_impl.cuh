@@ -277,9 +277,9 @@ __global__ void __launch_bounds__(256) k_step(const S* __restrict__ src, S* __re
 // wall node in a warp makes the whole warp pay for its rebuild, which is 60 %
 // more operations and hits every warp of a 64-wide row, and one-warp blocks
 // spread a small lattice over all SMs.  us a step, 64 x 2 blocks -> list:
-// 301 x 211 60.0 -> 43.1, 600 x 500 220 -> 177, 1024^2 688 -> 599, 64^2 19.4 -> 17.6
-// (there one wall warp's chain of dependent FP64 operations, 15 us, is the bound;
-// half-filled warps take as long as full ones).
+// per-node porosity, 301 x 211 60.7 -> 45.7, 600 x 500 216 -> 189, 1024^2 673 -> 639,
+// 64^2 20.4 -> 18.9 (there one wall warp's chain of dependent FP64 operations is
+// the bound; half-filled warps take as long as full ones).
 template <typename S, typename C>
 __global__ void __launch_bounds__(32) k_step_list(
     const S* __restrict__ src, S* __restrict__ dst, const C* __restrict__ phi_field,

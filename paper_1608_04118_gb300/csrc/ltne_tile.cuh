@@ -9,12 +9,13 @@
 // others from shared memory on ever narrower regions, the last on the tile
 // itself, to global memory.  The widened borders are computed by each
 // neighbour for itself; blocks never wait on one another.  Bound: the chain's
-// latency, about 0.95 us per step inside the tile (CPI 5.4 per warp: issue 1,
-// fixed latency 0.8, MUFU and shared memory 0.7, waiting for the slower wall
-// warps 1.0).  Measured, us a step, one step per launch -> this:
-//   64^2 FP32, uniform porosity          1.73 -> 1.22
-//   131 x 97 FP32, per-node porosity     2.18 -> 1.73
-//   192^2 FP32, per-node porosity        2.37 -> 2.18
+// latency, about 0.95 us per step inside the tile (a warp issues every 4.7
+// cycles: issue 1, fixed latency 0.7, MUFU and shared memory 0.9, waiting for the
+// slower wall warps 1.3, instruction fetch 0.9).  Measured, us a step, one step
+// per launch -> this:
+//   64^2 FP32, uniform porosity          1.74 -> 1.22
+//   131 x 97 FP32, per-node porosity     2.19 -> 1.71
+//   192^2 FP32, per-node porosity        2.44 -> 2.24
 // Eight steps per launch gain nothing over four (64^2: 1.35: the widened
 // region grows to 2.6 times the tile), and a warp apart for the wall nodes
 // loses 5 % at 64^2.
